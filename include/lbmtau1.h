@@ -168,17 +168,21 @@ int lbm_set_moments(lbm_ctx *ctx, const double *rho, const double *jx,
  * Enqueues nsteps LBMTau1 time steps (Algorithm 1), asynchronously.  The last
  * step of the call also reduces the residual and mass that lbm_residual
  * returns and checks for rho <= 0 or non-finite values.  nsteps = 0 is a
- * no-op.  On a stream that can be captured (not the legacy default stream,
- * and not under a capture of the caller's), runs of 16 inner steps are
- * replayed from a CUDA graph captured at first use (FP32 storage, or 16-bit
- * storage rounded to nearest; stochastic rounding launches every step).
+ * no-op.  The steps before the last are taken several per launch, unless a
+ * tile variant was set (lbm_set_variant), a side is shorter than 8 nodes or
+ * the step is the multiphase one: those take one launch per step, and on a
+ * stream that can be captured (not the legacy default stream, and not under a
+ * capture of the caller's) runs of 16 inner steps are then replayed from a
+ * CUDA graph captured at first use (FP32 storage, or 16-bit storage rounded
+ * to nearest; stochastic rounding launches every step).
  * Errors: LBM_E_INVAL (nsteps < 0), LBM_E_STATE, LBM_E_CUDA (launch failure).
  */
 int lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /*
  * Tile variant (block tile shape, 0 .. lbm_variant_count() - 1) of the
- * context's step kernel.  All variants give bit-identical states; they differ
+ * context's single-step kernel, which takes the reduced last step of a call
+ * and, once a variant is set by hand, every step.  All variants give bit-identical states; they differ
  * in how well their grid fills the device.  By default (variant -1) the first
  * step picks one from the domain size, the SM count and the kernels'
  * occupancy (the environment variable LBMTAU1_STEP_VARIANT, when set to a

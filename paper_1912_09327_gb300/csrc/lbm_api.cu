@@ -161,6 +161,8 @@ int lbm_create(const lbm_params *p, void *dev_workspace, size_t workspace_bytes,
   c->stream = static_cast<cudaStream_t>(cuda_stream);
   c->cur = 0;
   c->variant = -1;
+  c->variant_set = false;
+  for (bool &k : c->tiles_known) k = false;
   c->steps = 0;
   c->graph[0] = c->graph[1] = nullptr;
   c->graph_variant[0] = c->graph_variant[1] = -1;
@@ -430,7 +432,41 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   // the first step of each call (any one-time kernel set-up stays outside a
   // capture) and the reduced last step are launched directly.
   const bool graphs = !a.sr;
-  for (int64_t s = 0; s < nsteps;) {
+  int64_t s = 0;
+  // Several steps per launch up to the reduced last one (lbm_resident.cuh),
+  // unless the caller chose a tile variant of the single-step kernel.  Two
+  // inner steps at least: a launch for one costs what the kernel it replaces
+  // costs.
+  if (nsteps >= 3 && !c->variant_set && c->p.sc_g == 0.0) {
+    int64_t left = nsteps - 1;
+    const int run = static_cast<int>(left < lbmtau1::kLongRun
+                                         ? left : lbmtau1::kLongRun);
+    if (!c->tiles_known[run]) {
+      c->tiles[run] = lbmtau1::choose_resident(c->p.nx, c->p.ny, a.periodic_x,
+                                               a.periodic_y, run);
+      c->tiles_known[run] = true;
+    }
+    const lbmtau1::ResidentTiles &tiles = c->tiles[run];
+    // As few launches as the tiling allows, of nearly equal length, and as
+    // many as steps modulo two: the copy holding the state then alternates
+    // with the step count, as a caller's captured graph of an even number of
+    // steps relies on.
+    int64_t launches =
+        tiles.rows > 0 ? (left + tiles.steps - 1) / tiles.steps : 0;
+    if (launches > 0) launches += (left - launches) & 1;
+    for (; launches > 0; --launches) {
+      const int n = static_cast<int>((left + launches - 1) / launches);
+      a.src = c->f[c->cur];
+      a.dst = c->f[1 - c->cur];
+      a.step = static_cast<uint32_t>(c->steps + s);
+      cudaError_t e = lbmtau1::launch_resident(a, tiles, n, c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+      c->cur = 1 - c->cur;
+      s += n;
+      left -= n;
+    }
+  }
+  while (s < nsteps) {
     if (graphs && s >= 1 && nsteps - 1 - s >= kGraphChunk) {
       const int st = step_chunk(c, a);
       if (st) return st;
@@ -472,6 +508,7 @@ int lbm_set_variant(lbm_ctx *c, int32_t variant) {
   if (variant < -1 || variant >= lbmtau1::variant_count())
     return fail(c, LBM_E_INVAL, "variant %d out of range", int(variant));
   c->variant = variant;
+  c->variant_set = variant >= 0;
   return LBM_OK;
 }
 

@@ -18,6 +18,8 @@ inline bool stochastic_rounding(int storage, int rounding) {
          (rounding == LBM_ROUND_DEFAULT && storage != LBM_STORAGE_F32);
 }
 
+constexpr int kLongRun = 30;  // steps; the most one launch takes
+
 struct Layout {
   int64_t pitch = 0, staging_rows = 0, nblocks = 0;
   size_t field_bytes = 0;   // one field plane
@@ -47,6 +49,11 @@ struct lbm_ctx {
   cudaStream_t stream;
   int cur;              // copy holding the current state
   int variant;          // tile variant, chosen at the first step (-1 before)
+  bool variant_set;     // the caller chose the variant (lbm_set_variant)
+  // tilings of runs of 1 .. kLongRun steps (longer runs share the last one),
+  // each chosen at first use (tiles_known)
+  lbmtau1::ResidentTiles tiles[lbmtau1::kLongRun + 1];
+  bool tiles_known[lbmtau1::kLongRun + 1];
   int64_t steps;        // steps taken (seeds stochastic rounding)
   // 16 unreduced steps captured as one CUDA graph, one per starting copy
   // (rebuilt when the tile variant changes); none on an uncapturable stream

@@ -1676,13 +1676,5 @@ cudaError_t change_t(Fields now, Fields snap, const uint8_t *mask, int64_t nx,
   return cudaGetLastError();
 }
 
-// The launchers of storage type T, as the table lbm_step.cu dispatches on.
-template <typename T>
-constexpr StorageOps make_ops() {
-  return StorageOps{&launch_step_t<T>, &launch_batch_t<T>, &choose_variant_t<T>,
-                    &pack_t<T>,        &unpack_t<T>,       &solid_t<T>,
-                    &change_t<T>};
-}
-
 }  // namespace
 }  // namespace lbmtau1

@@ -1,0 +1,488 @@
+// Several LBMTau1 steps per launch on regions held in registers.
+//
+// What bounds one launch per step: small domains pay a launch and the serial
+// chain of a warp's marched rows (10 to 14 us a step from 64 x 32 to 1024^2,
+// where the arithmetic of all nodes is below 3 us), large ones the two trips
+// through memory (24 B a node).  Here a block loads a region of 64 columns x
+// (kR * warps) rows once, takes up to `steps` steps on it in registers and
+// stores the nodes that no missing neighbour has reached: a region's rim goes
+// stale by one node per step, so regions overlap by that much.  The inner
+// steps of lbm_step (all but its reduced last one) run this way.
+//
+// Layout: a lane holds two adjacent columns (one packed pair) of kR rows, a
+// warp all 64 columns.  Two columns and eight rows keep the same 16 nodes in a
+// lane as four columns and four rows, with half the temporaries per row: the
+// march over the rows fits 128 registers, so 16 warps are resident (the
+// single-step kernel holds 12).  Left and right neighbours come by shuffle;
+// what a warp's first and last row add to the warps below and above goes
+// through shared memory (double-buffered: one barrier a step), as sums, so no
+// row is computed twice.  No more than the node types' 9-bit wall codes and
+// those sums are in shared memory, and rows with no wall near take no branch
+// of the wall terms.
+//
+// Every node's arithmetic is that of step_tile (lbm_kernels.cuh), operation by
+// operation, and 16-bit formats round to storage after every step with the
+// random bits of the node's own place: the states are equal bit for bit.
+//
+// Measured (us per step, one launch per step -> this, periodic boxes, FP32):
+// 64^2 13.1 -> 0.7, 256^2 12.0 -> 0.9, 512^2 12.1 -> 1.5, 1024^2 14.2 -> 5.5,
+// 2048^2 40.7 -> 16.8, 4096^2 114 -> 62..75, 8192^2 311 -> 235.  A step on
+// full SMs runs at 480 k MLUPS before the overlap and the loads are paid for.
+#pragma once
+
+#include "lbm_kernels.cuh"
+
+namespace lbmtau1 {
+namespace {
+
+constexpr int kResCols = 2;                     // columns per lane
+constexpr int kResWidth = kLanes * kResCols;    // columns of a region
+constexpr int kResMaxWarps = 16;
+
+// What a warp hands its neighbours each step, one slot per lane: the sums a
+// boundary row adds to the row beyond it, and that row's momentum.
+struct alignas(16) EdgeA {
+  float2 dd, mx;
+};
+struct alignas(16) EdgeB {
+  float2 my, zx;
+};
+struct Edge {
+  EdgeA a[kLanes];
+  EdgeB b[kLanes];
+  float2 zy[kLanes];
+};
+
+template <int kR>
+__host__ __device__ constexpr int resident_smem(int warps) {
+  return 512 * static_cast<int>(sizeof(SolidSums)) +
+         warps * (4 * static_cast<int>(sizeof(Edge)) + kR * kLanes * 4);
+}
+
+// Programmatic dependent launch: wait until the launches before this one
+// have completed; let the next one start its prologue.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// One step's values of a column pair, rounded to the storage format and back
+// (exactly what a store and a load do).  (c0, c1): the domain's columns of
+// the pair, whose random bits are those of the pair they are stored in.
+template <typename T, bool kSr>
+__device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
+                                           uint32_t key, uint32_t c0,
+                                           uint32_t c1, bool aligned) {
+  using S = Storage<T>;
+  if constexpr (!std::is_same<T, float>::value) {
+    const float2 sd = bc(S::kD), sj = bc(S::kJ);
+    const float2 id = bc(1.0f / S::kD), ij = bc(1.0f / S::kJ);
+    union {
+      uint32_t w;
+      T e[2];
+    } u[3];
+    const float2 v[3] = {__fmul2_rn(d, sd), __fmul2_rn(x, sj),
+                         __fmul2_rn(y, sj)};
+    if constexpr (kSr) {
+      const uint32_t h0 = fmix32(key + (c0 & ~1u) * 0x9e3779b1u);
+#pragma unroll
+      for (int f = 0; f < 3; ++f)
+        u[f].w = pack_sr(T(), v[f].x, v[f].y,
+                         __funnelshift_l(h0, h0, 11 * f));
+      if (!aligned) {  // a wrapped pair of an odd width: column by column
+        const uint32_t h1 = fmix32(key + (c1 & ~1u) * 0x9e3779b1u);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          union {
+            uint32_t w;
+            T e[2];
+          } p, q;
+          p.w = pack_sr(T(), v[f].x, v[f].x, __funnelshift_l(h0, h0, 11 * f));
+          q.w = pack_sr(T(), v[f].y, v[f].y, __funnelshift_l(h1, h1, 11 * f));
+          u[f].e[0] = (c0 & 1u) ? p.e[1] : p.e[0];
+          u[f].e[1] = (c1 & 1u) ? q.e[1] : q.e[0];
+        }
+      }
+    } else {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        u[f].e[0] = S::encode(v[f].x);
+        u[f].e[1] = S::encode(v[f].y);
+      }
+    }
+    d = __fmul2_rn(make_float2(S::decode(u[0].e[0]), S::decode(u[0].e[1])), id);
+    x = __fmul2_rn(make_float2(S::decode(u[1].e[0]), S::decode(u[1].e[1])), ij);
+    y = __fmul2_rn(make_float2(S::decode(u[2].e[0]), S::decode(u[2].e[1])), ij);
+  }
+}
+
+template <typename T, int kR, bool kSr>
+__global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
+    lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
+  using S = Storage<T>;
+  constexpr bool kF32 = std::is_same<T, float>::value;
+  extern __shared__ __align__(128) unsigned char smem[];
+  SolidSums *lut = reinterpret_cast<SolidSums *>(smem);
+  const int warps = blockDim.x / kLanes;
+  Edge *edges = reinterpret_cast<Edge *>(smem + 512 * sizeof(SolidSums));
+  unsigned *codes = reinterpret_cast<unsigned *>(edges + 4 * warps);
+  const int lane = threadIdx.x & (kLanes - 1), w = threadIdx.x / kLanes;
+  build_solid_lut(lut);
+
+  // The region: its first column and row, and the outputs it owns.
+  const int bx = blockIdx.x, by = blockIdx.y;
+  const int nx = static_cast<int>(a.nx), ny = static_cast<int>(a.ny);
+  const int64_t pitch = a.pitch;
+  const int x0 = bx * g.ox - g.lead_x, y0 = by * g.oy - g.lead_y;
+  const int xb = x0 + kResCols * lane, yb = y0 + w * kR;
+  const int xlo = a.periodic_x || bx > 0 ? x0 + g.hx : 0;
+  const int xhi = a.periodic_x || bx + 1 < g.gx
+                      ? min(x0 + kResWidth - g.hx, nx) : nx;
+  const int ylo = a.periodic_y || by > 0 ? y0 + g.hy : 0;
+  const int yhi = a.periodic_y || by + 1 < g.gy
+                      ? min(y0 + warps * kR - g.hy, ny) : ny;
+
+  // columns of this lane in the domain (-1: outside)
+  auto wrap = [](int v, int n, int periodic) -> int {
+    if (v >= 0 && v < n) return v;
+    return periodic ? static_cast<int>(wrap_index(v, n)) : -1;
+  };
+  const int c0 = wrap(xb, nx, a.periodic_x), c1 = wrap(xb + 1, nx, a.periodic_x);
+  const bool aligned = (c0 & 1) == 0 && c1 == c0 + 1;
+  const bool vec = __all_sync(kFull, aligned && c0 >= 0);
+  const float fx = a.fx, fy = a.fy;
+
+  // Node types and fields of the region's rows (rows and columns outside the
+  // domain read some inside node and count as solid): all loads first, then
+  // what is derived from them.
+  const int q0 = max(c0, 0), q1 = max(c1, 0);
+  unsigned m0[kR + 2], m1[kR + 2];  // rows yb - 1 .. yb + kR
+  int64_t off[kR + 2];
+  unsigned inside = 0u;
+#pragma unroll
+  for (int r = 0; r < kR + 2; ++r) {
+    const int row = wrap(yb + r - 1, ny, a.periodic_y);
+    inside |= (row >= 0 ? 1u : 0u) << r;
+    off[r] = static_cast<int64_t>(max(row, 0)) * pitch;
+  }
+  if (vec) {
+#pragma unroll
+    for (int r = 0; r < kR + 2; ++r)
+      m0[r] = *reinterpret_cast<const unsigned short *>(a.mask + off[r] + q0);
+#pragma unroll
+    for (int r = 0; r < kR + 2; ++r) {
+      m1[r] = m0[r] >> 8;
+      m0[r] &= 0xffu;
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < kR + 2; ++r) {
+      m0[r] = a.mask[off[r] + q0];
+      m1[r] = a.mask[off[r] + q1];
+    }
+  }
+  pdl_wait();  // the fields: written by the launch before this one
+  float2 d[kR], zx[kR], zy[kR];
+  const T *sd = static_cast<const T *>(a.src.d);
+  const T *sx = static_cast<const T *>(a.src.jx);
+  const T *sy = static_cast<const T *>(a.src.jy);
+  if (vec) {
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      float2 t[1];
+      load_pairs<2, T>(sd + off[r + 1] + q0, t, 1.0f / S::kD);
+      d[r] = t[0];
+      load_pairs<2, T>(sx + off[r + 1] + q0, t, 1.0f / S::kJ);
+      zx[r] = t[0];
+      load_pairs<2, T>(sy + off[r + 1] + q0, t, 1.0f / S::kJ);
+      zy[r] = t[0];
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const int64_t o = off[r + 1];
+      d[r] = make_float2(S::decode(sd[o + q0]) * (1.0f / S::kD),
+                         S::decode(sd[o + q1]) * (1.0f / S::kD));
+      zx[r] = make_float2(S::decode(sx[o + q0]) * (1.0f / S::kJ),
+                          S::decode(sx[o + q1]) * (1.0f / S::kJ));
+      zy[r] = make_float2(S::decode(sy[o + q0]) * (1.0f / S::kJ),
+                          S::decode(sy[o + q1]) * (1.0f / S::kJ));
+    }
+  }
+  unsigned walls = 0u, keep = 0u;  // rows with solid neighbours / kept nodes
+  unsigned any = 0u;
+#pragma unroll
+  for (int r = 0; r < kR + 2; ++r) any |= m0[r] | m1[r];
+  any |= (c0 < 0 || c1 < 0 || inside != (1u << (kR + 2)) - 1u) ? 1u : 0u;
+  if (__any_sync(kFull, any != 0u)) {
+    // solid bits of a row's columns -1 .. 2, and its fluid bits
+    auto types = [&](int r, unsigned &fluid) -> unsigned {
+      const bool in = (inside >> r) & 1u;
+      const unsigned t0 = in && c0 >= 0 ? m0[r] : 1u;
+      const unsigned t1 = in && c1 >= 0 ? m1[r] : 1u;
+      fluid = (t0 == 0u ? 1u : 0u) | (t1 == 0u ? 2u : 0u);
+      const unsigned s = (t0 == 1u ? 1u : 0u) | (t1 == 1u ? 2u : 0u);
+      const unsigned l = __shfl_up_sync(kFull, s, 1);
+      const unsigned p = __shfl_down_sync(kFull, s, 1);
+      return (l >> 1) | (s << 1) | ((p & 1u) << 3);
+    };
+    unsigned fl, fc, fn;
+    unsigned lo = types(0, fl), own = types(1, fc);
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const unsigned hi = types(r + 2, fn);
+      const unsigned i0 = (lo & 7u) | ((own & 7u) << 3) | ((hi & 7u) << 6);
+      const unsigned i1 = (lo >> 1) | ((own >> 1) << 3) | ((hi >> 1) << 6);
+      codes[(w * kR + r) * kLanes + lane] = i0 | (i1 << 9) | (fc << 18);
+      if (__any_sync(kFull, (lo | own | hi) != 0u)) walls |= 1u << r;
+      if (__any_sync(kFull, fc != 3u)) keep |= 1u << r;
+      // a solid node's momentum as a source: -F (zero momentum j + F)
+      if (own & 2u) { d[r].x = 0.f; zx[r].x = -fx; zy[r].x = -fy; }
+      if (own & 4u) { d[r].y = 0.f; zx[r].y = -fx; zy[r].y = -fy; }
+      lo = own;
+      own = hi;
+      fc = fn;
+    }
+  }
+  __syncthreads();
+  pdl_release();
+
+  const float2 F2x = bc(fx), F2y = bc(fy), F22y = bc(2.0f * fy);
+  const float2 one = bc(1.0f), c3 = bc(3.0f), cm15 = bc(-1.5f);
+  const float2 w1_9 = bc(k1_9), w1_36 = bc(k1_36), w1_12 = bc(k1_12),
+               w1_3 = bc(k1_3), w4_9 = bc(k4_9), w1_6 = bc(k1_6),
+               wm1_6 = bc(-k1_6), half = bc(0.5f), mhalf = bc(-0.5f),
+               quarter = bc(0.25f);
+
+  for (int t = 0; t < nsteps; ++t) {
+    const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
+    const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
+    Edge *mine = edges + ((t & 1) * warps + w) * 2;  // [0] down, [1] up
+
+    // completes row r: acc holds South(r - 1) + Same(r) with the vertical
+    // difference to row r - 1, (nd, nx_, ny_) the row above's contribution
+    // and (ex, ey) its momentum less the row's own
+    auto finish = [&](int r, float2 ad, float2 ax, float2 ay, float2 nd,
+                      float2 nmx, float2 nmy, float2 ex, float2 ey) {
+      const float2 dO = d[r], zxO = zx[r], zyO = zy[r];
+      float2 dn = add(ad, nd);
+      float2 incx = fma2(w1_6, ex, add(add(ax, nmx), F2x));
+      float2 incy = fma2(half, ey, add(add(ay, nmy), F2y));
+      unsigned code = 0u;
+      if (((walls | keep) >> r) & 1u)
+        code = codes[(w * kR + r) * kLanes + lane];
+      if ((walls >> r) & 1u) {
+        const SolidSums E0 = lut[code & 511u], E1 = lut[(code >> 9) & 511u];
+        dn.x = fmaf(dO.x, E0.s0, dn.x);
+        incx.x = fmaf(dO.x, E0.sx, incx.x);
+        incy.x = fmaf(dO.x, E0.sy, incy.x);
+        dn.y = fmaf(dO.y, E1.s0, dn.y);
+        incx.y = fmaf(dO.y, E1.sx, incx.y);
+        incy.y = fmaf(dO.y, E1.sy, incy.y);
+      }
+      if constexpr (kF32 && kSr) {
+        incx = fma2(lead_pow2(zxO), dither, incx);
+        incy = fma2(lead_pow2(zyO), dither, incy);
+      }
+      float2 xn = add(zxO, incx), yn = add(zyO, incy);
+      if constexpr (!kF32) {
+        int row = yb + r;
+        if constexpr (kSr)
+          if (a.periodic_y) row = wrap(row, ny, 1);
+        round_pair<T, kSr>(
+            dn, xn, yn,
+            fmix32(step_key ^ (static_cast<uint32_t>(row) * 0x85ebca77u)),
+            static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), aligned);
+      }
+      if ((keep >> r) & 1u) {
+        const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
+        dn = make_float2(f0 ? dn.x : dO.x, f1 ? dn.y : dO.y);
+        xn = make_float2(f0 ? xn.x : zxO.x, f1 ? xn.y : zxO.y);
+        yn = make_float2(f0 ? yn.x : zyO.x, f1 ? yn.y : zyO.y);
+      }
+      d[r] = dn;
+      zx[r] = xn;
+      zy[r] = yn;
+    };
+
+    float2 acd, acx, acy;              // South(r - 1) + Same(r)
+    float2 td, tx, ty;                 // South(r)
+    float2 s0d, s0x;                   // Same(0)
+    float2 n1d, n1x, n1y, e1x, e1y;    // North(1) and z(1) - z(0)
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const float2 dc = d[r], zxC = zx[r], zyC = zy[r];
+      const float2 mx = add(zxC, F2x), my = add(zyC, F2y);
+      const float2 rho = add(dc, one);
+      const float2 ir =
+          make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+      const float2 q = mul(mx, ir);
+      const float2 pxx = mul(q, mx), pxy = mul(q, my);
+      const float2 pyy = mul(mul(my, my), ir);
+      const float2 tr = add(pxx, pyy);
+      const float2 K = fma2(w1_9, dc, fma2(w1_3, pxx, mul(wm1_6, pyy)));
+      const float2 P = fma2(c3, pyy, fma2(cm15, pxx, dc));
+      const float2 G = fma2(w1_12, tr, mul(w1_36, dc));
+      const float2 X = mul(quarter, pxy);
+      const float2 R0 = fma2(cm15, tr, dc);
+      struct Halo {
+        float m, p;
+      };
+      auto halo = [&](float2 v) -> Halo {
+        return {__shfl_up_sync(kFull, v.y, 1), __shfl_down_sync(kFull, v.x, 1)};
+      };
+      const Halo hK = halo(K), hG = halo(G), hX = halo(X);
+      const Halo hZx = halo(zxC), hZy = halo(zyC);
+      auto lpr = [](float2 v, Halo h) {
+        return make_float2(__fadd_rn(h.m, v.y), __fadd_rn(v.x, h.p));
+      };
+      auto lmr = [](float2 v, Halo h) {
+        return make_float2(__fsub_rn(h.m, v.y), __fsub_rn(v.x, h.p));
+      };
+      // (left - own) + (right - own), both differences exact
+      auto second = [](float2 v, Halo h) {
+        const float e = __fsub_rn(v.y, v.x);
+        return make_float2(__fadd_rn(__fsub_rn(h.m, v.x), e),
+                           __fsub_rn(__fsub_rn(h.p, v.y), e));
+      };
+      const float2 Ks = lpr(K, hK), Kd = lmr(K, hK);
+      const float2 Gs = lpr(G, hG), Gd = lmr(G, hG);
+      const float2 Xs = lpr(X, hX), Xd = lmr(X, hX);
+      const float2 mxd = lmr(zxC, hZx), myd = lmr(zyC, hZy);
+      const float2 mys = add(lpr(zyC, hZy), F22y);
+      const float2 hx = second(zxC, hZx), hy = second(zyC, hZy);
+      const float2 U = fma2(w1_9, P, fma2(w1_12, mxd, Gs));
+      const float2 V = fma2(w1_3, my, fma2(w1_12, mys, Xd));
+      const float2 Y = fma2(w1_12, hy, Xd);
+      const float2 Up = fma2(w1_12, hx, Gd), Vp = fma2(w1_12, myd, Xs);
+      const float2 Sdd = fma2(w4_9, R0, fma2(w1_3, mxd, Ks));
+      const float2 Smx = fma2(w1_3, hx, Kd);
+      const float2 nd = sub(U, V), nmx = sub(Up, Vp), nmy = sub(Y, U);
+      if (r == 0) {
+        mine[0].a[lane] = {nd, nmx};
+        mine[0].b[lane] = {nmy, zxC};
+        mine[0].zy[lane] = zyC;
+        s0d = Sdd;
+        s0x = Smx;
+      } else {
+        const float2 ex = sub(zxC, zx[r - 1]), ey = sub(zyC, zy[r - 1]);
+        const float2 bd = add(td, Sdd);
+        const float2 bx_ = fma2(wm1_6, ex, add(tx, Smx));
+        const float2 by_ = fma2(mhalf, ey, ty);
+        if (r == 1) {
+          n1d = nd;
+          n1x = nmx;
+          n1y = nmy;
+          e1x = ex;
+          e1y = ey;
+        } else {
+          finish(r - 1, acd, acx, acy, nd, nmx, nmy, ex, ey);
+        }
+        acd = bd;
+        acx = bx_;
+        acy = by_;
+      }
+      td = add(U, V);
+      tx = add(Up, Vp);
+      ty = add(Y, U);
+      if (r == kR - 1) {
+        mine[1].a[lane] = {td, tx};
+        mine[1].b[lane] = {ty, zxC};
+        mine[1].zy[lane] = zyC;
+      }
+    }
+    __syncthreads();
+    {  // the first row, with the row below's contribution (none: solid)
+      EdgeA ea = {bc(0.f), bc(0.f)};
+      EdgeB eb = {bc(0.f), bc(-fx)};
+      float2 ez = bc(-fy);
+      if (w > 0) {
+        const Edge *e = mine - 1;
+        ea = e->a[lane];
+        eb = e->b[lane];
+        ez = e->zy[lane];
+      }
+      // the last row's momentum may be overwritten by row 0's when kR == 1
+      finish(0, add(ea.dd, s0d),
+             fma2(w1_6, sub(eb.zx, zx[0]), add(ea.mx, s0x)),
+             fma2(half, sub(ez, zy[0]), eb.my), n1d, n1x, n1y, e1x, e1y);
+    }
+    {  // the last row, with the row above's contribution
+      EdgeA ea = {bc(0.f), bc(0.f)};
+      EdgeB eb = {bc(0.f), bc(-fx)};
+      float2 ez = bc(-fy);
+      if (w + 1 < warps) {
+        const Edge *e = mine + 2;
+        ea = e->a[lane];
+        eb = e->b[lane];
+        ez = e->zy[lane];
+      }
+      finish(kR - 1, acd, acx, acy, ea.dd, ea.mx, eb.my,
+             sub(eb.zx, zx[kR - 1]), sub(ez, zy[kR - 1]));
+    }
+  }
+
+  // the owned outputs
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    const int row = yb + r;
+    if (row < ylo || row >= yhi || xb < xlo || xb >= xhi) continue;
+    const int64_t o = static_cast<int64_t>(row) * pitch + xb;
+    const float2 vd[1] = {d[r]}, vx[1] = {zx[r]}, vy[1] = {zy[r]};
+    store_pairs<2, T>(static_cast<T *>(a.dst.d) + o, vd, S::kD);
+    store_pairs<2, T>(static_cast<T *>(a.dst.jx) + o, vx, S::kJ);
+    store_pairs<2, T>(static_cast<T *>(a.dst.jy) + o, vy, S::kJ);
+  }
+}
+
+template <typename T, int kR, bool kSr>
+cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
+                              int nsteps, cudaStream_t s) {
+  auto kern = lbm_resident_kernel<T, kR, kSr>;
+  static cudaError_t attr = cudaFuncSetAttribute(
+      kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      resident_smem<kR>(kResMaxWarps));
+  if (attr != cudaSuccess) return attr;
+  (void)cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.gx, g.gy);
+  cfg.blockDim = dim3(g.warps * kLanes);
+  cfg.dynamicSmemBytes = resident_smem<kR>(g.warps);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a, g, nsteps);
+}
+
+template <typename T>
+cudaError_t launch_resident_t(const StepLaunch &a, const ResidentTiles &g,
+                              int nsteps, cudaStream_t s) {
+  if (a.sr) {
+    switch (g.rows) {
+      case 2: return launch_resident_k<T, 2, true>(a, g, nsteps, s);
+      case 4: return launch_resident_k<T, 4, true>(a, g, nsteps, s);
+      default: return launch_resident_k<T, 8, true>(a, g, nsteps, s);
+    }
+  }
+  switch (g.rows) {
+    case 2: return launch_resident_k<T, 2, false>(a, g, nsteps, s);
+    case 4: return launch_resident_k<T, 4, false>(a, g, nsteps, s);
+    default: return launch_resident_k<T, 8, false>(a, g, nsteps, s);
+  }
+}
+
+// The launchers of storage type T, as the table lbm_step.cu dispatches on.
+template <typename T>
+constexpr StorageOps make_ops() {
+  return StorageOps{&launch_step_t<T>, &launch_batch_t<T>, &choose_variant_t<T>,
+                    &launch_resident_t<T>, &pack_t<T>,     &unpack_t<T>,
+                    &solid_t<T>,       &change_t<T>};
+}
+
+}  // namespace
+}  // namespace lbmtau1

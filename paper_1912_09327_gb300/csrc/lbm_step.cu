@@ -1,5 +1,7 @@
 // Dispatch of the LBMTau1 step kernels over the storage formats, and the
 // kernels that do not depend on the format (tile flags, reductions).
+#include <math.h>
+
 #include "lbm_kernels.cuh"
 
 namespace lbmtau1 {
@@ -210,6 +212,108 @@ cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s) {
   if (a.ny >= (int64_t(1) << 30) || a.nx >= (int64_t(1) << 30))
     return cudaErrorInvalidValue;  // the tile loop indexes rows in 32 bits
   return ops(a.storage).step(a, reduce, s);
+}
+
+// Tiling with `rows` rows per warp, `warps` warps and `steps` steps a launch.
+static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
+                                    int periodic_y, int rows, int warps,
+                                    int steps) {
+  constexpr int kWidth = 64;
+  ResidentTiles g;
+  const int height = rows * warps;
+  g.rows = rows;
+  g.warps = warps;
+  g.steps = steps;
+  g.hx = (steps + 1) & ~1;
+  g.hy = steps;
+  g.ox = kWidth - 2 * g.hx;
+  g.oy = height - 2 * g.hy;
+  if (!periodic_x) {
+    // one lane of outside columns before the domain, one column after it
+    g.lead_x = 2;
+    if (nx <= kWidth - 3) {
+      g.hx = 0;
+      g.gx = 1;
+    } else if (g.ox > 0) {
+      g.gx = static_cast<int>((nx + 2 - (kWidth - 1) + g.ox - 1) / g.ox) + 1;
+    }
+  } else if (g.ox > 0) {
+    g.lead_x = g.hx;
+    g.gx = static_cast<int>((nx + g.ox - 1) / g.ox);
+  }
+  if (!periodic_y) {
+    if (ny <= height) {
+      g.hy = 0;
+      g.gy = 1;
+    } else if (g.oy > 0) {
+      g.gy = static_cast<int>((ny - height + g.oy - 1) / g.oy) + 1;
+    }
+  } else if (g.oy > 0) {
+    g.lead_y = g.hy;
+    g.gy = static_cast<int>((ny + g.oy - 1) / g.oy);
+  }
+  if (g.gx <= 0 || g.gy <= 0 || g.gy > 65535) g.rows = 0;
+  return g;
+}
+
+ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
+                              int periodic_y, int nsteps) {
+  ResidentTiles best;
+  if (nx < 8 || ny < 8 || nsteps < 1 || forced_variant() >= 0) return best;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
+            cudaSuccess)
+      n = 0;
+    return n;
+  }();
+  if (sms <= 0) return best;
+  constexpr int kWarpsPerSm = 16;
+  // time of one step on an SM whose resident warps hold `rows` rows of 64
+  // columns: 3300 nodes/us once 16 warps are there, and at least the chain
+  // of a warp's own r rows
+  auto step_us = [](int r, int rows) {
+    return fmax(0.0195 * rows + 0.18, 0.20 + 0.12 * r);
+  };
+  // The tiling with the shortest expected time per step.  A launch of t steps
+  // pays for its loads and stores once, so that small domains want long
+  // launches; a region loses t rows and columns of outputs on every side it
+  // shares, so that domains of many regions want short ones (4 steps on
+  // 64 x 64 regions from about 1500^2 on).  Fitted to launches on a GB300
+  // (64^2 .. 8192^2 boxes): within 13 % of the best of the swept tilings.
+  double best_us = 0.0;
+  for (int r = 2; r <= 8; r *= 2)
+    for (int w = 1; w <= kWarpsPerSm; ++w)
+      for (int t = 1; t <= nsteps; ++t) {
+        const ResidentTiles g =
+            resident_tiles(nx, ny, periodic_x, periodic_y, r, w, t);
+        if (g.rows == 0) continue;
+        const int64_t blocks = static_cast<int64_t>(g.gx) * g.gy;
+        const int64_t per_sm = (blocks + sms - 1) / sms;
+        const int c = kWarpsPerSm / w;
+        // k blocks on an SM at a time; their loads and stores overlap with
+        // other blocks' steps only when more blocks follow
+        auto round_us = [&](int64_t k) {
+          const int rows = static_cast<int>(k) * r * ((w + 3) / 4 * 4);
+          const double over = 1.5 + 0.03 * rows;
+          return t * step_us(r, rows) +
+                 (per_sm > k && k > 1 ? 0.4 : 1.0) * over;
+        };
+        double us = static_cast<double>(per_sm / c) * round_us(c);
+        if (per_sm % c) us += round_us(per_sm % c);
+        us /= t;
+        if (best.rows == 0 || us < best_us) {
+          best = g;
+          best_us = us;
+        }
+      }
+  return best;
+}
+
+cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
+                            int nsteps, cudaStream_t s) {
+  return ops(a.storage).resident(a, g, nsteps, s);
 }
 
 cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,

@@ -80,6 +80,18 @@ struct BatchLaunch {
   unsigned int *done;     // blocks finished in this launch (zero between)
 };
 
+// Tiling of a launch that takes several steps on register-resident regions
+// of 64 columns x (rows * warps) rows (lbm_resident.cuh): region (bx, by)
+// starts at column bx * ox - lead_x and row by * oy - lead_y and owns the
+// nodes at least (hx, hy) inside its sides that face other regions.
+struct ResidentTiles {
+  int rows = 0;    // rows per warp (2, 4 or 8); 0: no such launch
+  int warps = 0;   // warps per block (stacked in y)
+  int steps = 0;   // steps a launch may take
+  int gx = 0, gy = 0;
+  int ox = 0, oy = 0, hx = 0, hy = 0, lead_x = 0, lead_y = 0;
+};
+
 // The launchers of one storage format.  The kernels are templates on the
 // storage type, instantiated once per format in its own translation unit
 // (lbm_step_f32.cu, lbm_step_f16.cu, lbm_step_bf16.cu); the entry points
@@ -89,6 +101,8 @@ struct StorageOps {
   cudaError_t (*batch)(int v, const BatchLaunch &b, bool reduce,
                        cudaStream_t s);
   int (*choose)(int64_t nx, int64_t ny);
+  cudaError_t (*resident)(const StepLaunch &a, const ResidentTiles &g,
+                          int nsteps, cudaStream_t s);
   cudaError_t (*pack)(const double *staging, Fields f, int64_t nx,
                       int64_t pitch, int64_t y0, int64_t rows,
                       cudaStream_t s);
@@ -152,6 +166,15 @@ cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,
 // Enqueues one step; `reduce` also writes block partials of
 // (sum |du|^2, sum |u|^2, sum (rho - 1)) and raises the flag on instability.
 cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s);
+
+// Tiling for a run of nsteps steps on an nx x ny domain (rows = 0: none; the
+// steps are then launched one by one).
+ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
+                              int periodic_y, int nsteps);
+
+// Enqueues nsteps <= g.steps unreduced steps from a.src to a.dst.
+cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
+                            int nsteps, cudaStream_t s);
 
 // Sums the partial triples of `nblocks` block tiles (kTileWarps each, added
 // in warp order per block) in FP64 in a fixed order into out[0..2].

@@ -17,8 +17,11 @@
 // what a warp's first and last row add to the warps below and above goes
 // through shared memory (double-buffered: one barrier a step), as sums, so no
 // row is computed twice.  No more than the node types' 9-bit wall codes and
-// those sums are in shared memory, and rows with no wall near take no branch
-// of the wall terms.
+// those sums are in shared memory.  The time loop exists twice: a block with no
+// wall and no kept node in or around its rows takes the copy without the wall
+// terms' tests and branches (4096^2 box: 62 -> 52.6 us a step; the tests cost
+// issue slots, and their code instruction fetches: 1.07 no-instruction stalls
+// per issue before, 0.24 after).
 //
 // Every node's arithmetic is that of step_tile (lbm_kernels.cuh), operation by
 // operation, and 16-bit formats round to storage after every step with the
@@ -26,8 +29,9 @@
 //
 // Measured (us per step, one launch per step -> this, periodic boxes, FP32):
 // 64^2 13.1 -> 0.7, 256^2 12.0 -> 0.9, 512^2 12.1 -> 1.5, 1024^2 14.2 -> 5.5,
-// 2048^2 40.7 -> 16.8, 4096^2 114 -> 62..75, 8192^2 311 -> 235.  A step on
-// full SMs runs at 480 k MLUPS before the overlap and the loads are paid for.
+// 2048^2 40.7 -> 14.5, 4096^2 114 -> 52.6.  A step on full SMs runs at 500 k
+// MLUPS before the overlap and the loads are paid for; the FMA pipe, which a
+// packed operation holds for two cycles, is then 68 % busy.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -66,6 +70,13 @@ __device__ __forceinline__ void pdl_wait() {
 }
 __device__ __forceinline__ void pdl_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// 1 / x as __fdividef(1, x) rounds it, without the product by one.
+__device__ __forceinline__ float rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // One step's values of a column pair, rounded to the storage format and back
@@ -246,7 +257,7 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
       fc = fn;
     }
   }
-  __syncthreads();
+  const bool any_walls = __syncthreads_or((walls | keep) != 0u);
   pdl_release();
 
   const float2 F2x = bc(fx), F2y = bc(fy), F22y = bc(2.0f * fy);
@@ -256,6 +267,9 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
                wm1_6 = bc(-k1_6), half = bc(0.5f), mhalf = bc(-0.5f),
                quarter = bc(0.25f);
 
+  // kWalls: some row of the block has solid neighbours or kept nodes
+  auto march = [&](auto with_walls) {
+  constexpr bool kWalls = decltype(with_walls)::value;
   for (int t = 0; t < nsteps; ++t) {
     const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
     const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
@@ -271,9 +285,9 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
       float2 incx = fma2(w1_6, ex, add(add(ax, nmx), F2x));
       float2 incy = fma2(half, ey, add(add(ay, nmy), F2y));
       unsigned code = 0u;
-      if (((walls | keep) >> r) & 1u)
+      if (kWalls && (((walls | keep) >> r) & 1u))
         code = codes[(w * kR + r) * kLanes + lane];
-      if ((walls >> r) & 1u) {
+      if (kWalls && ((walls >> r) & 1u)) {
         const SolidSums E0 = lut[code & 511u], E1 = lut[(code >> 9) & 511u];
         dn.x = fmaf(dO.x, E0.s0, dn.x);
         incx.x = fmaf(dO.x, E0.sx, incx.x);
@@ -296,7 +310,7 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
             fmix32(step_key ^ (static_cast<uint32_t>(row) * 0x85ebca77u)),
             static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), aligned);
       }
-      if ((keep >> r) & 1u) {
+      if (kWalls && ((keep >> r) & 1u)) {
         const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
         dn = make_float2(f0 ? dn.x : dO.x, f1 ? dn.y : dO.y);
         xn = make_float2(f0 ? xn.x : zxO.x, f1 ? xn.y : zxO.y);
@@ -316,8 +330,7 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
       const float2 dc = d[r], zxC = zx[r], zyC = zy[r];
       const float2 mx = add(zxC, F2x), my = add(zyC, F2y);
       const float2 rho = add(dc, one);
-      const float2 ir =
-          make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+      const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
       const float2 q = mul(mx, ir);
       const float2 pxx = mul(q, mx), pxy = mul(q, my);
       const float2 pyy = mul(mul(my, my), ir);
@@ -404,7 +417,6 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
         eb = e->b[lane];
         ez = e->zy[lane];
       }
-      // the last row's momentum may be overwritten by row 0's when kR == 1
       finish(0, add(ea.dd, s0d),
              fma2(w1_6, sub(eb.zx, zx[0]), add(ea.mx, s0x)),
              fma2(half, sub(ez, zy[0]), eb.my), n1d, n1x, n1y, e1x, e1y);
@@ -423,6 +435,11 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
              sub(eb.zx, zx[kR - 1]), sub(ez, zy[kR - 1]));
     }
   }
+  };
+  if (any_walls)
+    march(std::true_type{});
+  else
+    march(std::false_type{});
 
   // the owned outputs
 #pragma unroll

@@ -28,10 +28,10 @@
 // random bits of the node's own place: the states are equal bit for bit.
 //
 // Measured (us per step, one launch per step -> this, periodic boxes, FP32):
-// 64^2 13.1 -> 0.7, 256^2 12.0 -> 0.9, 512^2 12.1 -> 1.5, 1024^2 14.2 -> 5.5,
-// 2048^2 40.7 -> 14.5, 4096^2 114 -> 52.6.  A step on full SMs runs at 500 k
-// MLUPS before the overlap and the loads are paid for; the FMA pipe, which a
-// packed operation holds for two cycles, is then 68 % busy.
+// 64^2 13.1 -> 0.64, 256^2 12.0 -> 0.84, 512^2 12.1 -> 1.34, 1024^2 14.2 -> 4.5,
+// 2048^2 40.7 -> 13.7, 4096^2 114 -> 50.7, 8192^2 312 -> 194.  A step on full
+// SMs runs at 500 k MLUPS before the overlap and the loads are paid for; the
+// FMA pipe, which a packed operation holds for two cycles, is 72 % busy then.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -140,7 +140,6 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   Edge *edges = reinterpret_cast<Edge *>(smem + 512 * sizeof(SolidSums));
   unsigned *codes = reinterpret_cast<unsigned *>(edges + 4 * warps);
   const int lane = threadIdx.x & (kLanes - 1), w = threadIdx.x / kLanes;
-  build_solid_lut(lut);
 
   // The region: its first column and row, and the outputs it owns.
   const int bx = blockIdx.x, by = blockIdx.y;
@@ -165,61 +164,102 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   const bool vec = __all_sync(kFull, aligned && c0 >= 0);
   const float fx = a.fx, fy = a.fy;
 
-  // Node types and fields of the region's rows (rows and columns outside the
-  // domain read some inside node and count as solid): all loads first, then
-  // what is derived from them.
-  const int q0 = max(c0, 0), q1 = max(c1, 0);
+  // Node types and fields of the region's rows: all loads first, then what is
+  // derived from them.  A region that lies in the domain with the rows around
+  // it needs no index of its own per row and column: one 32-bit offset per row
+  // serves the four planes (a 64-bit index per row, column and plane took 7 %
+  // of the instructions of a four-step launch: box 4096^2 52.6 -> 50.7 us a
+  // step, 64 x 32 regions 69 -> 59).
   unsigned m0[kR + 2], m1[kR + 2];  // rows yb - 1 .. yb + kR
-  int64_t off[kR + 2];
-  unsigned inside = 0u;
-#pragma unroll
-  for (int r = 0; r < kR + 2; ++r) {
-    const int row = wrap(yb + r - 1, ny, a.periodic_y);
-    inside |= (row >= 0 ? 1u : 0u) << r;
-    off[r] = static_cast<int64_t>(max(row, 0)) * pitch;
-  }
-  if (vec) {
+  unsigned inside = (1u << (kR + 2)) - 1u;
+  float2 d[kR], zx[kR], zy[kR];
+  const T *sd = static_cast<const T *>(a.src.d);
+  const T *sx = static_cast<const T *>(a.src.jx);
+  const T *sy = static_cast<const T *>(a.src.jy);
+  // (its blocks with walls build their table below)
+  const bool inner = x0 >= 0 && x0 + kResWidth <= nx && y0 >= 1 &&
+                     y0 + warps * kR < ny;
+  const int64_t corner = static_cast<int64_t>(y0) * pitch + x0;
+  const unsigned step_y = static_cast<unsigned>(pitch);
+  const unsigned mine0 = static_cast<unsigned>(w * kR) * step_y +
+                         static_cast<unsigned>(kResCols * lane);
+  if (inner) {
+    const uint8_t *pm = a.mask + (corner - pitch);
 #pragma unroll
     for (int r = 0; r < kR + 2; ++r)
-      m0[r] = *reinterpret_cast<const unsigned short *>(a.mask + off[r] + q0);
+      m0[r] = *reinterpret_cast<const unsigned short *>(pm + (mine0 + r * step_y));
+    pdl_wait();  // the fields: written by the launch before this one
+    sd += corner;
+    sx += corner;
+    sy += corner;
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      const unsigned o = mine0 + r * step_y;
+      float2 t[1];
+      load_pairs<2, T>(sd + o, t, 1.0f / S::kD);
+      d[r] = t[0];
+      load_pairs<2, T>(sx + o, t, 1.0f / S::kJ);
+      zx[r] = t[0];
+      load_pairs<2, T>(sy + o, t, 1.0f / S::kJ);
+      zy[r] = t[0];
+    }
 #pragma unroll
     for (int r = 0; r < kR + 2; ++r) {
       m1[r] = m0[r] >> 8;
       m0[r] &= 0xffu;
     }
   } else {
+    // rows and columns outside the domain read some inside node and count as
+    // solid
+    build_solid_lut(lut);
+    const int q0 = max(c0, 0), q1 = max(c1, 0);
+    int64_t off[kR + 2];
+    inside = 0u;
 #pragma unroll
     for (int r = 0; r < kR + 2; ++r) {
-      m0[r] = a.mask[off[r] + q0];
-      m1[r] = a.mask[off[r] + q1];
+      const int row = wrap(yb + r - 1, ny, a.periodic_y);
+      inside |= (row >= 0 ? 1u : 0u) << r;
+      off[r] = static_cast<int64_t>(max(row, 0)) * pitch;
     }
-  }
-  pdl_wait();  // the fields: written by the launch before this one
-  float2 d[kR], zx[kR], zy[kR];
-  const T *sd = static_cast<const T *>(a.src.d);
-  const T *sx = static_cast<const T *>(a.src.jx);
-  const T *sy = static_cast<const T *>(a.src.jy);
-  if (vec) {
+    if (vec) {
 #pragma unroll
-    for (int r = 0; r < kR; ++r) {
-      float2 t[1];
-      load_pairs<2, T>(sd + off[r + 1] + q0, t, 1.0f / S::kD);
-      d[r] = t[0];
-      load_pairs<2, T>(sx + off[r + 1] + q0, t, 1.0f / S::kJ);
-      zx[r] = t[0];
-      load_pairs<2, T>(sy + off[r + 1] + q0, t, 1.0f / S::kJ);
-      zy[r] = t[0];
+      for (int r = 0; r < kR + 2; ++r)
+        m0[r] = *reinterpret_cast<const unsigned short *>(a.mask + off[r] + q0);
+#pragma unroll
+      for (int r = 0; r < kR + 2; ++r) {
+        m1[r] = m0[r] >> 8;
+        m0[r] &= 0xffu;
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < kR + 2; ++r) {
+        m0[r] = a.mask[off[r] + q0];
+        m1[r] = a.mask[off[r] + q1];
+      }
     }
-  } else {
+    pdl_wait();  // the fields: written by the launch before this one
+    if (vec) {
 #pragma unroll
-    for (int r = 0; r < kR; ++r) {
-      const int64_t o = off[r + 1];
-      d[r] = make_float2(S::decode(sd[o + q0]) * (1.0f / S::kD),
-                         S::decode(sd[o + q1]) * (1.0f / S::kD));
-      zx[r] = make_float2(S::decode(sx[o + q0]) * (1.0f / S::kJ),
-                          S::decode(sx[o + q1]) * (1.0f / S::kJ));
-      zy[r] = make_float2(S::decode(sy[o + q0]) * (1.0f / S::kJ),
-                          S::decode(sy[o + q1]) * (1.0f / S::kJ));
+      for (int r = 0; r < kR; ++r) {
+        float2 t[1];
+        load_pairs<2, T>(sd + off[r + 1] + q0, t, 1.0f / S::kD);
+        d[r] = t[0];
+        load_pairs<2, T>(sx + off[r + 1] + q0, t, 1.0f / S::kJ);
+        zx[r] = t[0];
+        load_pairs<2, T>(sy + off[r + 1] + q0, t, 1.0f / S::kJ);
+        zy[r] = t[0];
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const int64_t o = off[r + 1];
+        d[r] = make_float2(S::decode(sd[o + q0]) * (1.0f / S::kD),
+                           S::decode(sd[o + q1]) * (1.0f / S::kD));
+        zx[r] = make_float2(S::decode(sx[o + q0]) * (1.0f / S::kJ),
+                            S::decode(sx[o + q1]) * (1.0f / S::kJ));
+        zy[r] = make_float2(S::decode(sy[o + q0]) * (1.0f / S::kJ),
+                            S::decode(sy[o + q1]) * (1.0f / S::kJ));
+      }
     }
   }
   unsigned walls = 0u, keep = 0u;  // rows with solid neighbours / kept nodes
@@ -259,6 +299,10 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   }
   const bool any_walls = __syncthreads_or((walls | keep) != 0u);
   pdl_release();
+  if (any_walls && inner) {
+    build_solid_lut(lut);
+    __syncthreads();
+  }
 
   const float2 F2x = bc(fx), F2y = bc(fy), F22y = bc(2.0f * fy);
   const float2 one = bc(1.0f), c3 = bc(3.0f), cm15 = bc(-1.5f);
@@ -269,172 +313,172 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
 
   // kWalls: some row of the block has solid neighbours or kept nodes
   auto march = [&](auto with_walls) {
-  constexpr bool kWalls = decltype(with_walls)::value;
-  for (int t = 0; t < nsteps; ++t) {
-    const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
-    const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
-    Edge *mine = edges + ((t & 1) * warps + w) * 2;  // [0] down, [1] up
+    constexpr bool kWalls = decltype(with_walls)::value;
+    for (int t = 0; t < nsteps; ++t) {
+      const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
+      const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
+      Edge *mine = edges + ((t & 1) * warps + w) * 2;  // [0] down, [1] up
 
-    // completes row r: acc holds South(r - 1) + Same(r) with the vertical
-    // difference to row r - 1, (nd, nx_, ny_) the row above's contribution
-    // and (ex, ey) its momentum less the row's own
-    auto finish = [&](int r, float2 ad, float2 ax, float2 ay, float2 nd,
-                      float2 nmx, float2 nmy, float2 ex, float2 ey) {
-      const float2 dO = d[r], zxO = zx[r], zyO = zy[r];
-      float2 dn = add(ad, nd);
-      float2 incx = fma2(w1_6, ex, add(add(ax, nmx), F2x));
-      float2 incy = fma2(half, ey, add(add(ay, nmy), F2y));
-      unsigned code = 0u;
-      if (kWalls && (((walls | keep) >> r) & 1u))
-        code = codes[(w * kR + r) * kLanes + lane];
-      if (kWalls && ((walls >> r) & 1u)) {
-        const SolidSums E0 = lut[code & 511u], E1 = lut[(code >> 9) & 511u];
-        dn.x = fmaf(dO.x, E0.s0, dn.x);
-        incx.x = fmaf(dO.x, E0.sx, incx.x);
-        incy.x = fmaf(dO.x, E0.sy, incy.x);
-        dn.y = fmaf(dO.y, E1.s0, dn.y);
-        incx.y = fmaf(dO.y, E1.sx, incx.y);
-        incy.y = fmaf(dO.y, E1.sy, incy.y);
-      }
-      if constexpr (kF32 && kSr) {
-        incx = fma2(lead_pow2(zxO), dither, incx);
-        incy = fma2(lead_pow2(zyO), dither, incy);
-      }
-      float2 xn = add(zxO, incx), yn = add(zyO, incy);
-      if constexpr (!kF32) {
-        int row = yb + r;
-        if constexpr (kSr)
-          if (a.periodic_y) row = wrap(row, ny, 1);
-        round_pair<T, kSr>(
-            dn, xn, yn,
-            fmix32(step_key ^ (static_cast<uint32_t>(row) * 0x85ebca77u)),
-            static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), aligned);
-      }
-      if (kWalls && ((keep >> r) & 1u)) {
-        const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
-        dn = make_float2(f0 ? dn.x : dO.x, f1 ? dn.y : dO.y);
-        xn = make_float2(f0 ? xn.x : zxO.x, f1 ? xn.y : zxO.y);
-        yn = make_float2(f0 ? yn.x : zyO.x, f1 ? yn.y : zyO.y);
-      }
-      d[r] = dn;
-      zx[r] = xn;
-      zy[r] = yn;
-    };
-
-    float2 acd, acx, acy;              // South(r - 1) + Same(r)
-    float2 td, tx, ty;                 // South(r)
-    float2 s0d, s0x;                   // Same(0)
-    float2 n1d, n1x, n1y, e1x, e1y;    // North(1) and z(1) - z(0)
-#pragma unroll
-    for (int r = 0; r < kR; ++r) {
-      const float2 dc = d[r], zxC = zx[r], zyC = zy[r];
-      const float2 mx = add(zxC, F2x), my = add(zyC, F2y);
-      const float2 rho = add(dc, one);
-      const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
-      const float2 q = mul(mx, ir);
-      const float2 pxx = mul(q, mx), pxy = mul(q, my);
-      const float2 pyy = mul(mul(my, my), ir);
-      const float2 tr = add(pxx, pyy);
-      const float2 K = fma2(w1_9, dc, fma2(w1_3, pxx, mul(wm1_6, pyy)));
-      const float2 P = fma2(c3, pyy, fma2(cm15, pxx, dc));
-      const float2 G = fma2(w1_12, tr, mul(w1_36, dc));
-      const float2 X = mul(quarter, pxy);
-      const float2 R0 = fma2(cm15, tr, dc);
-      struct Halo {
-        float m, p;
-      };
-      auto halo = [&](float2 v) -> Halo {
-        return {__shfl_up_sync(kFull, v.y, 1), __shfl_down_sync(kFull, v.x, 1)};
-      };
-      const Halo hK = halo(K), hG = halo(G), hX = halo(X);
-      const Halo hZx = halo(zxC), hZy = halo(zyC);
-      auto lpr = [](float2 v, Halo h) {
-        return make_float2(__fadd_rn(h.m, v.y), __fadd_rn(v.x, h.p));
-      };
-      auto lmr = [](float2 v, Halo h) {
-        return make_float2(__fsub_rn(h.m, v.y), __fsub_rn(v.x, h.p));
-      };
-      // (left - own) + (right - own), both differences exact
-      auto second = [](float2 v, Halo h) {
-        const float e = __fsub_rn(v.y, v.x);
-        return make_float2(__fadd_rn(__fsub_rn(h.m, v.x), e),
-                           __fsub_rn(__fsub_rn(h.p, v.y), e));
-      };
-      const float2 Ks = lpr(K, hK), Kd = lmr(K, hK);
-      const float2 Gs = lpr(G, hG), Gd = lmr(G, hG);
-      const float2 Xs = lpr(X, hX), Xd = lmr(X, hX);
-      const float2 mxd = lmr(zxC, hZx), myd = lmr(zyC, hZy);
-      const float2 mys = add(lpr(zyC, hZy), F22y);
-      const float2 hx = second(zxC, hZx), hy = second(zyC, hZy);
-      const float2 U = fma2(w1_9, P, fma2(w1_12, mxd, Gs));
-      const float2 V = fma2(w1_3, my, fma2(w1_12, mys, Xd));
-      const float2 Y = fma2(w1_12, hy, Xd);
-      const float2 Up = fma2(w1_12, hx, Gd), Vp = fma2(w1_12, myd, Xs);
-      const float2 Sdd = fma2(w4_9, R0, fma2(w1_3, mxd, Ks));
-      const float2 Smx = fma2(w1_3, hx, Kd);
-      const float2 nd = sub(U, V), nmx = sub(Up, Vp), nmy = sub(Y, U);
-      if (r == 0) {
-        mine[0].a[lane] = {nd, nmx};
-        mine[0].b[lane] = {nmy, zxC};
-        mine[0].zy[lane] = zyC;
-        s0d = Sdd;
-        s0x = Smx;
-      } else {
-        const float2 ex = sub(zxC, zx[r - 1]), ey = sub(zyC, zy[r - 1]);
-        const float2 bd = add(td, Sdd);
-        const float2 bx_ = fma2(wm1_6, ex, add(tx, Smx));
-        const float2 by_ = fma2(mhalf, ey, ty);
-        if (r == 1) {
-          n1d = nd;
-          n1x = nmx;
-          n1y = nmy;
-          e1x = ex;
-          e1y = ey;
-        } else {
-          finish(r - 1, acd, acx, acy, nd, nmx, nmy, ex, ey);
+      // completes row r: acc holds South(r - 1) + Same(r) with the vertical
+      // difference to row r - 1, (nd, nx_, ny_) the row above's contribution
+      // and (ex, ey) its momentum less the row's own
+      auto finish = [&](int r, float2 ad, float2 ax, float2 ay, float2 nd,
+                        float2 nmx, float2 nmy, float2 ex, float2 ey) {
+        const float2 dO = d[r], zxO = zx[r], zyO = zy[r];
+        float2 dn = add(ad, nd);
+        float2 incx = fma2(w1_6, ex, add(add(ax, nmx), F2x));
+        float2 incy = fma2(half, ey, add(add(ay, nmy), F2y));
+        unsigned code = 0u;
+        if (kWalls && (((walls | keep) >> r) & 1u))
+          code = codes[(w * kR + r) * kLanes + lane];
+        if (kWalls && ((walls >> r) & 1u)) {
+          const SolidSums E0 = lut[code & 511u], E1 = lut[(code >> 9) & 511u];
+          dn.x = fmaf(dO.x, E0.s0, dn.x);
+          incx.x = fmaf(dO.x, E0.sx, incx.x);
+          incy.x = fmaf(dO.x, E0.sy, incy.x);
+          dn.y = fmaf(dO.y, E1.s0, dn.y);
+          incx.y = fmaf(dO.y, E1.sx, incx.y);
+          incy.y = fmaf(dO.y, E1.sy, incy.y);
         }
-        acd = bd;
-        acx = bx_;
-        acy = by_;
+        if constexpr (kF32 && kSr) {
+          incx = fma2(lead_pow2(zxO), dither, incx);
+          incy = fma2(lead_pow2(zyO), dither, incy);
+        }
+        float2 xn = add(zxO, incx), yn = add(zyO, incy);
+        if constexpr (!kF32) {
+          int row = yb + r;
+          if constexpr (kSr)
+            if (a.periodic_y) row = wrap(row, ny, 1);
+          round_pair<T, kSr>(
+              dn, xn, yn,
+              fmix32(step_key ^ (static_cast<uint32_t>(row) * 0x85ebca77u)),
+              static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), aligned);
+        }
+        if (kWalls && ((keep >> r) & 1u)) {
+          const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
+          dn = make_float2(f0 ? dn.x : dO.x, f1 ? dn.y : dO.y);
+          xn = make_float2(f0 ? xn.x : zxO.x, f1 ? xn.y : zxO.y);
+          yn = make_float2(f0 ? yn.x : zyO.x, f1 ? yn.y : zyO.y);
+        }
+        d[r] = dn;
+        zx[r] = xn;
+        zy[r] = yn;
+      };
+
+      float2 acd, acx, acy;              // South(r - 1) + Same(r)
+      float2 td, tx, ty;                 // South(r)
+      float2 s0d, s0x;                   // Same(0)
+      float2 n1d, n1x, n1y, e1x, e1y;    // North(1) and z(1) - z(0)
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const float2 dc = d[r], zxC = zx[r], zyC = zy[r];
+        const float2 mx = add(zxC, F2x), my = add(zyC, F2y);
+        const float2 rho = add(dc, one);
+        const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
+        const float2 q = mul(mx, ir);
+        const float2 pxx = mul(q, mx), pxy = mul(q, my);
+        const float2 pyy = mul(mul(my, my), ir);
+        const float2 tr = add(pxx, pyy);
+        const float2 K = fma2(w1_9, dc, fma2(w1_3, pxx, mul(wm1_6, pyy)));
+        const float2 P = fma2(c3, pyy, fma2(cm15, pxx, dc));
+        const float2 G = fma2(w1_12, tr, mul(w1_36, dc));
+        const float2 X = mul(quarter, pxy);
+        const float2 R0 = fma2(cm15, tr, dc);
+        struct Halo {
+          float m, p;
+        };
+        auto halo = [&](float2 v) -> Halo {
+          return {__shfl_up_sync(kFull, v.y, 1), __shfl_down_sync(kFull, v.x, 1)};
+        };
+        const Halo hK = halo(K), hG = halo(G), hX = halo(X);
+        const Halo hZx = halo(zxC), hZy = halo(zyC);
+        auto lpr = [](float2 v, Halo h) {
+          return make_float2(__fadd_rn(h.m, v.y), __fadd_rn(v.x, h.p));
+        };
+        auto lmr = [](float2 v, Halo h) {
+          return make_float2(__fsub_rn(h.m, v.y), __fsub_rn(v.x, h.p));
+        };
+        // (left - own) + (right - own), both differences exact
+        auto second = [](float2 v, Halo h) {
+          const float e = __fsub_rn(v.y, v.x);
+          return make_float2(__fadd_rn(__fsub_rn(h.m, v.x), e),
+                             __fsub_rn(__fsub_rn(h.p, v.y), e));
+        };
+        const float2 Ks = lpr(K, hK), Kd = lmr(K, hK);
+        const float2 Gs = lpr(G, hG), Gd = lmr(G, hG);
+        const float2 Xs = lpr(X, hX), Xd = lmr(X, hX);
+        const float2 mxd = lmr(zxC, hZx), myd = lmr(zyC, hZy);
+        const float2 mys = add(lpr(zyC, hZy), F22y);
+        const float2 hx = second(zxC, hZx), hy = second(zyC, hZy);
+        const float2 U = fma2(w1_9, P, fma2(w1_12, mxd, Gs));
+        const float2 V = fma2(w1_3, my, fma2(w1_12, mys, Xd));
+        const float2 Y = fma2(w1_12, hy, Xd);
+        const float2 Up = fma2(w1_12, hx, Gd), Vp = fma2(w1_12, myd, Xs);
+        const float2 Sdd = fma2(w4_9, R0, fma2(w1_3, mxd, Ks));
+        const float2 Smx = fma2(w1_3, hx, Kd);
+        const float2 nd = sub(U, V), nmx = sub(Up, Vp), nmy = sub(Y, U);
+        if (r == 0) {
+          mine[0].a[lane] = {nd, nmx};
+          mine[0].b[lane] = {nmy, zxC};
+          mine[0].zy[lane] = zyC;
+          s0d = Sdd;
+          s0x = Smx;
+        } else {
+          const float2 ex = sub(zxC, zx[r - 1]), ey = sub(zyC, zy[r - 1]);
+          const float2 bd = add(td, Sdd);
+          const float2 bx_ = fma2(wm1_6, ex, add(tx, Smx));
+          const float2 by_ = fma2(mhalf, ey, ty);
+          if (r == 1) {
+            n1d = nd;
+            n1x = nmx;
+            n1y = nmy;
+            e1x = ex;
+            e1y = ey;
+          } else {
+            finish(r - 1, acd, acx, acy, nd, nmx, nmy, ex, ey);
+          }
+          acd = bd;
+          acx = bx_;
+          acy = by_;
+        }
+        td = add(U, V);
+        tx = add(Up, Vp);
+        ty = add(Y, U);
+        if (r == kR - 1) {
+          mine[1].a[lane] = {td, tx};
+          mine[1].b[lane] = {ty, zxC};
+          mine[1].zy[lane] = zyC;
+        }
       }
-      td = add(U, V);
-      tx = add(Up, Vp);
-      ty = add(Y, U);
-      if (r == kR - 1) {
-        mine[1].a[lane] = {td, tx};
-        mine[1].b[lane] = {ty, zxC};
-        mine[1].zy[lane] = zyC;
+      __syncthreads();
+      {  // the first row, with the row below's contribution (none: solid)
+        EdgeA ea = {bc(0.f), bc(0.f)};
+        EdgeB eb = {bc(0.f), bc(-fx)};
+        float2 ez = bc(-fy);
+        if (w > 0) {
+          const Edge *e = mine - 1;
+          ea = e->a[lane];
+          eb = e->b[lane];
+          ez = e->zy[lane];
+        }
+        finish(0, add(ea.dd, s0d),
+               fma2(w1_6, sub(eb.zx, zx[0]), add(ea.mx, s0x)),
+               fma2(half, sub(ez, zy[0]), eb.my), n1d, n1x, n1y, e1x, e1y);
+      }
+      {  // the last row, with the row above's contribution
+        EdgeA ea = {bc(0.f), bc(0.f)};
+        EdgeB eb = {bc(0.f), bc(-fx)};
+        float2 ez = bc(-fy);
+        if (w + 1 < warps) {
+          const Edge *e = mine + 2;
+          ea = e->a[lane];
+          eb = e->b[lane];
+          ez = e->zy[lane];
+        }
+        finish(kR - 1, acd, acx, acy, ea.dd, ea.mx, eb.my,
+               sub(eb.zx, zx[kR - 1]), sub(ez, zy[kR - 1]));
       }
     }
-    __syncthreads();
-    {  // the first row, with the row below's contribution (none: solid)
-      EdgeA ea = {bc(0.f), bc(0.f)};
-      EdgeB eb = {bc(0.f), bc(-fx)};
-      float2 ez = bc(-fy);
-      if (w > 0) {
-        const Edge *e = mine - 1;
-        ea = e->a[lane];
-        eb = e->b[lane];
-        ez = e->zy[lane];
-      }
-      finish(0, add(ea.dd, s0d),
-             fma2(w1_6, sub(eb.zx, zx[0]), add(ea.mx, s0x)),
-             fma2(half, sub(ez, zy[0]), eb.my), n1d, n1x, n1y, e1x, e1y);
-    }
-    {  // the last row, with the row above's contribution
-      EdgeA ea = {bc(0.f), bc(0.f)};
-      EdgeB eb = {bc(0.f), bc(-fx)};
-      float2 ez = bc(-fy);
-      if (w + 1 < warps) {
-        const Edge *e = mine + 2;
-        ea = e->a[lane];
-        eb = e->b[lane];
-        ez = e->zy[lane];
-      }
-      finish(kR - 1, acd, acx, acy, ea.dd, ea.mx, eb.my,
-             sub(eb.zx, zx[kR - 1]), sub(ez, zy[kR - 1]));
-    }
-  }
   };
   if (any_walls)
     march(std::true_type{});
@@ -442,15 +486,20 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     march(std::false_type{});
 
   // the owned outputs
+  if (xb < xlo || xb >= xhi) return;
+  const int64_t first = static_cast<int64_t>(y0) * pitch + x0;
+  T *dd = static_cast<T *>(a.dst.d) + first;
+  T *dx = static_cast<T *>(a.dst.jx) + first;
+  T *dy = static_cast<T *>(a.dst.jy) + first;
 #pragma unroll
   for (int r = 0; r < kR; ++r) {
     const int row = yb + r;
-    if (row < ylo || row >= yhi || xb < xlo || xb >= xhi) continue;
-    const int64_t o = static_cast<int64_t>(row) * pitch + xb;
+    if (row < ylo || row >= yhi) continue;
+    const int64_t o = static_cast<int64_t>(mine0 + r * step_y);
     const float2 vd[1] = {d[r]}, vx[1] = {zx[r]}, vy[1] = {zy[r]};
-    store_pairs<2, T>(static_cast<T *>(a.dst.d) + o, vd, S::kD);
-    store_pairs<2, T>(static_cast<T *>(a.dst.jx) + o, vx, S::kJ);
-    store_pairs<2, T>(static_cast<T *>(a.dst.jy) + o, vy, S::kJ);
+    store_pairs<2, T>(dd + o, vd, S::kD);
+    store_pairs<2, T>(dx + o, vx, S::kJ);
+    store_pairs<2, T>(dy + o, vy, S::kJ);
   }
 }
 

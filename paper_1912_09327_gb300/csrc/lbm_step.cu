@@ -259,7 +259,10 @@ static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
 ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
                               int periodic_y, int nsteps) {
   ResidentTiles best;
-  if (nx < 8 || ny < 8 || nsteps < 1 || forced_variant() >= 0) return best;
+  // rows wrap at most once, and a region's offsets fit 32 bits
+  if (nx < 8 || ny < 8 || nx > (1 << 23) || nsteps < 1 ||
+      forced_variant() >= 0)
+    return best;
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -271,17 +274,17 @@ ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
   if (sms <= 0) return best;
   constexpr int kWarpsPerSm = 16;
   // time of one step on an SM whose resident warps hold `rows` rows of 64
-  // columns: 3300 nodes/us once 16 warps are there, and at least the chain
+  // columns: 3400 nodes/us once 16 warps are there, and at least the chain
   // of a warp's own r rows
   auto step_us = [](int r, int rows) {
-    return fmax(0.0195 * rows + 0.18, 0.20 + 0.12 * r);
+    return fmax(0.0188 * rows + 0.1, 0.18 + 0.1 * r);
   };
   // The tiling with the shortest expected time per step.  A launch of t steps
   // pays for its loads and stores once, so that small domains want long
   // launches; a region loses t rows and columns of outputs on every side it
-  // shares, so that domains of many regions want short ones (4 steps on
+  // shares, so that domains of many regions want short ones (3 or 4 steps on
   // 64 x 64 regions from about 1500^2 on).  Fitted to launches on a GB300
-  // (64^2 .. 8192^2 boxes): within 13 % of the best of the swept tilings.
+  // (64^2 .. 8192^2 boxes).
   double best_us = 0.0;
   for (int r = 2; r <= 8; r *= 2)
     for (int w = 1; w <= kWarpsPerSm; ++w)
@@ -292,13 +295,15 @@ ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
         const int64_t blocks = static_cast<int64_t>(g.gx) * g.gy;
         const int64_t per_sm = (blocks + sms - 1) / sms;
         const int c = kWarpsPerSm / w;
-        // k blocks on an SM at a time; their loads and stores overlap with
-        // other blocks' steps only when more blocks follow
+        // k blocks on an SM at a time (four schedulers: warps count by
+        // fours); where more blocks follow, their loads and stores overlap
+        // with each other's steps
         auto round_us = [&](int64_t k) {
           const int rows = static_cast<int>(k) * r * ((w + 3) / 4 * 4);
-          const double over = 1.5 + 0.03 * rows;
-          return t * step_us(r, rows) +
-                 (per_sm > k && k > 1 ? 0.4 : 1.0) * over;
+          const double steps = t * step_us(r, rows);
+          const double over = 1.3 + 0.02 * rows;
+          return steps + (per_sm > k && k > 1
+                              ? fmax(0.25 * over, over - 0.42 * steps) : over);
         };
         double us = static_cast<double>(per_sm / c) * round_us(c);
         if (per_sm % c) us += round_us(per_sm % c);

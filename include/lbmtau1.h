@@ -330,15 +330,15 @@ int lbm_step_noalloc(const float *drho_in, const float *jx_in,
 void lbm_destroy(lbm_ctx *ctx);
 
 /*
- * Batches: one launch per time step for many independent domains.
+ * Batches: shared launches for many independent domains.
  *
  * The paper steps one domain at a time; independent domains (Algorithm 1
  * applied to each) can share a launch.  A batch references existing contexts
  * (each with its own workspace, geometry and state) that use the batch's
- * stream.  lbm_batch_step advances every member by nsteps with one launch per
- * step over a work list of all members' block tiles, taken by a persistent
- * grid through an atomic counter; runs of steps inside a call are replayed
- * from a captured CUDA graph.  Each member ends bit for bit where it would
+ * stream.  lbm_batch_step advances every member by nsteps: the steps before the
+ * last several per launch, over a list of all members' regions; the reduced
+ * last step over a work list of all members' block tiles, taken by a
+ * persistent grid through an atomic counter.  Each member ends bit for bit where it would
  * have ended alone, and afterwards lbm_moments / lbm_residual / lbm_step work
  * on it as usual (the last step of the call is reduced for every member).
  */
@@ -372,7 +372,8 @@ int32_t lbm_batch_members(const lbm_batch *b);
  * LBM_E_CUDA. */
 int lbm_batch_step(lbm_batch *b, int64_t nsteps);
 
-/* Tile variants (block tile shapes) of the step kernels: their count, and
+/* Tile variants (block tile shapes) of the single-step kernels, which a batch
+ * uses for the reduced last step of a call: their count, and
  * the one a batch uses (set by hand or by lbm_batch_autotune; the default is
  * variant 0 unless LBMTAU1_STEP_VARIANT names another).  All variants give
  * bit-identical states. */

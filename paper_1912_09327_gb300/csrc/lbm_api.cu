@@ -442,8 +442,9 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
     const int run = static_cast<int>(left < lbmtau1::kLongRun
                                          ? left : lbmtau1::kLongRun);
     if (!c->tiles_known[run]) {
-      c->tiles[run] = lbmtau1::choose_resident(c->p.nx, c->p.ny, a.periodic_x,
-                                               a.periodic_y, run);
+      const lbmtau1::ResidentShape d = {c->p.nx, c->p.ny, a.periodic_x,
+                                        a.periodic_y};
+      c->tiles[run] = lbmtau1::choose_resident(&d, 1, run);
       c->tiles_known[run] = true;
     }
     const lbmtau1::ResidentTiles &tiles = c->tiles[run];

@@ -5,10 +5,18 @@
 // partials); the batch holds a device table of member descriptors and a work
 // list of block tiles (member, tile x, tile y).  A persistent grid walks the
 // list through an atomic counter, so small and large domains share the GPU in
-// one launch instead of one under-filled launch per domain.  Runs of steps
-// between the first and the last step of a call are replayed from a CUDA
-// graph of kChunk steps.  Each tile runs the same code as the single-domain
-// kernel, so a member's state is bit for bit the one it would reach alone.
+// one launch instead of one under-filled launch per domain.  Each tile runs
+// the same code as the single-domain kernel, so a member's state is bit for bit
+// the one it would reach alone.
+//
+// That is the reduced last step of a call.  The steps before it are taken
+// several per launch on the members' register-resident regions
+// (lbm_resident.cuh), one block per region, all members' in one launch: 48
+// domains of the mix (7.7 M nodes) went from 87 to 37 us a step, where one
+// launch per step was bound by the issue of the general tile code.  Only
+// where the regions do not serve (a side below 8 nodes, a forced tile variant,
+// a list larger than the workspace) is there one launch per step, replayed
+// from a CUDA graph of kChunk steps.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
@@ -34,7 +42,7 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct BatchLayout {
   size_t off_members = 0, off_items = 0, off_nitems = 0, off_counters = 0;
-  size_t off_gather = 0;
+  size_t off_gather = 0, off_regions = 0;
   size_t total = 0;
 };
 
@@ -53,6 +61,10 @@ BatchLayout batch_layout(int32_t capacity, int64_t max_tiles) {
   off += align_up(sizeof(unsigned) * (kChunk + 3), kAlign);
   L.off_gather = off;
   off += align_up(sizeof(double) * 4 * static_cast<size_t>(capacity), kAlign);
+  L.off_regions = off;
+  off += align_up(sizeof(int4) * static_cast<size_t>(max_tiles) *
+                      lbmtau1::kTileWarps,
+                  kAlign);
   L.total = off;
   return L;
 }
@@ -70,6 +82,14 @@ struct lbm_batch {
   uint32_t clock;        // host mirror of the batch clock
   bool clock_set;        // device clock and done count zeroed
   double *d_gather;      // 4 doubles per member: result sums and flag
+  // The regions of the multi-step launches: those of members that round to
+  // nearest, then those that round stochastically.  Rebuilt with the work
+  // list, or when a call's length asks for another tiling (regions_for).
+  int4 *d_regions;
+  std::vector<int4> h_regions;
+  int nregions[2];
+  lbmtau1::ResidentTiles tiles;  // rows 0: one launch per step
+  int regions_for;
   cudaStream_t stream;
   std::vector<lbm_ctx *> slots;
   std::vector<BatchMember> h_members;
@@ -107,9 +127,53 @@ void drop_graph(lbm_batch *b) {
   b->graph_variant = -1;
 }
 
+// The longest run whose own length decides the tiling of the regions.
+constexpr int kBatchRun = 8;
+
+// Chooses the tiling for runs of `run` steps and uploads the members' regions
+// (b->tiles.rows = 0 when the steps have to be launched one by one: sizes the
+// regions do not serve, or a workspace too small for their list).
+int build_regions(lbm_batch *b, int run) {
+  const int n = static_cast<int>(b->packed.size());
+  std::vector<lbmtau1::ResidentShape> shapes(n);
+  for (int i = 0; i < n; ++i) {
+    const BatchMember &m = b->h_members[i];
+    shapes[i] = {m.nx, m.ny, m.periodic_x, m.periodic_y};
+  }
+  b->regions_for = run;
+  b->nregions[0] = b->nregions[1] = 0;
+  b->tiles = lbmtau1::choose_resident(shapes.data(), n, run);
+  if (b->tiles.rows == 0) return LBM_OK;
+  b->h_regions.clear();
+  const size_t most =
+      static_cast<size_t>(b->max_tiles) * lbmtau1::kTileWarps;
+  for (int sr = 0; sr < 2; ++sr)
+    for (int i = 0; i < n; ++i) {
+      BatchMember &m = b->h_members[i];
+      if ((m.sr != 0) != (sr != 0)) continue;
+      const lbmtau1::ResidentTiles g = lbmtau1::resident_tiles(
+          shapes[i], b->tiles.rows, b->tiles.warps, b->tiles.steps);
+      const size_t count = static_cast<size_t>(g.gx) * g.gy;
+      if (b->h_regions.size() + count > most) {
+        b->tiles.rows = 0;
+        return LBM_OK;
+      }
+      for (int y = 0; y < g.gy; ++y)
+        for (int x = 0; x < g.gx; ++x)
+          b->h_regions.push_back(make_int4(i, x, y, 0));
+      b->nregions[sr] += static_cast<int>(count);
+    }
+  cudaError_t e = cudaMemcpyAsync(b->d_regions, b->h_regions.data(),
+                                  sizeof(int4) * b->h_regions.size(),
+                                  cudaMemcpyHostToDevice, b->stream);
+  if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(regions)");
+  return LBM_OK;
+}
+
 // Refreshes the member table (every call: a member may have been stepped on
 // its own since) and, when membership or the variant changed, the work list.
-int upload(lbm_batch *b) {
+// `run`: steps the call takes before its last one (0: none).
+int upload(lbm_batch *b, int64_t run) {
   b->packed.clear();
   for (lbm_ctx *c : b->slots)
     if (c) b->packed.push_back(c);
@@ -210,6 +274,19 @@ int upload(lbm_batch *b) {
                                     cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(nitems)");
     b->items_dirty = false;
+    b->regions_for = 0;
+  }
+  if (n && run >= 2) {
+    const int r = static_cast<int>(run < kBatchRun ? run : kBatchRun);
+    if (b->regions_for != r) {
+      const int st = build_regions(b, r);
+      if (st) return st;
+    }
+    if (b->tiles.rows > 0)
+      for (BatchMember &m : b->h_members)
+        m.tiles = lbmtau1::resident_tiles(
+            {m.nx, m.ny, m.periodic_x, m.periodic_y}, b->tiles.rows,
+            b->tiles.warps, b->tiles.steps);
   }
   if (n) {
     cudaError_t e = cudaMemcpyAsync(b->d_members, b->h_members.data(),
@@ -347,6 +424,9 @@ int lbm_batch_create(int32_t capacity, int64_t max_tiles, void *dev_workspace,
   b->d_nitems = reinterpret_cast<int *>(base + L.off_nitems);
   b->d_counters = reinterpret_cast<unsigned *>(base + L.off_counters);
   b->d_gather = reinterpret_cast<double *>(base + L.off_gather);
+  b->d_regions = reinterpret_cast<int4 *>(base + L.off_regions);
+  b->nregions[0] = b->nregions[1] = 0;
+  b->regions_for = 0;
   b->stream = static_cast<cudaStream_t>(cuda_stream);
   b->clock = 0;
   b->clock_set = false;
@@ -423,7 +503,7 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
   if (!b) return LBM_E_INVAL;
   if (nsteps < 0) return bfail(b, LBM_E_INVAL, "nsteps < 0");
   if (nsteps == 0 || lbm_batch_members(b) == 0) return LBM_OK;
-  int st = upload(b);
+  int st = upload(b, nsteps - 1);
   if (st) return st;
   if (!b->clock_set) {  // the batch clock and the done count start at zero
     cudaError_t e = cudaMemsetAsync(b->d_counters + kChunk + 1, 0,
@@ -432,12 +512,42 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
     b->clock_set = true;
   }
   int64_t s = 0;
+  // The steps before the last: several per launch, as lbm_step takes them
+  // (as many launches as steps modulo two, so that the copies' parity below
+  // is the step count's).
+  if (nsteps >= 3 && b->tiles.rows > 0) {
+    int64_t left = nsteps - 1;
+    int64_t launches = (left + b->tiles.steps - 1) / b->tiles.steps;
+    launches += (left - launches) & 1;
+    for (int64_t l = 0; l < launches; ++l) {
+      const int n =
+          static_cast<int>((left + launches - l - 1) / (launches - l));
+      lbmtau1::ResidentBatch r;
+      r.members = b->d_members;
+      r.rows = b->tiles.rows;
+      r.warps = b->tiles.warps;
+      r.storage = b->storage;
+      r.parity = static_cast<int>(l & 1);
+      r.clock = b->clock + static_cast<uint32_t>(s);
+      r.next_clock = b->d_counters + kChunk + 1;
+      for (int sr = 0; sr < 2; ++sr) {
+        if (b->nregions[sr] == 0) continue;
+        r.items = b->d_regions + (sr ? b->nregions[0] : 0);
+        r.nitems = b->nregions[sr];
+        r.sr = sr;
+        cudaError_t e = lbmtau1::launch_resident_batch(r, n, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "batch region launch");
+      }
+      left -= n;
+      s += n;
+    }
+  }
   // first step direct (one-time kernel set-up stays outside any capture)
   for (; s < nsteps && s < 2; ++s) {
     st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1);
     if (st) return st;
   }
-  while (s + kChunk <= nsteps - 1) {
+  while ((s & 1) == 0 && s + kChunk <= nsteps - 1) {
     st = graph_chunk(b);
     if (st) return st;
     s += kChunk;
@@ -513,7 +623,7 @@ int lbm_batch_residuals(lbm_batch *b, double *residual, double *mass,
     residual[i] = mass[i] = 0.0;
     status[i] = LBM_E_STATE;
   }
-  int st = upload(b);  // descriptors in slot order of the current members
+  int st = upload(b, 0);  // descriptors in slot order of the current members
   if (st) return st;
   const int n = static_cast<int>(b->packed.size());
   if (n == 0) return LBM_OK;

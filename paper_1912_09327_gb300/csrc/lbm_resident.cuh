@@ -129,12 +129,14 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
   }
 }
 
+// Takes nsteps steps on region (bx, by); every thread of the block calls it.
 template <typename T, int kR, bool kSr>
-__global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
-    lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
+__device__ __forceinline__ void resident_region(const StepLaunch &a,
+                                                const ResidentTiles &g, int bx,
+                                                int by, int nsteps,
+                                                unsigned char *smem) {
   using S = Storage<T>;
   constexpr bool kF32 = std::is_same<T, float>::value;
-  extern __shared__ __align__(128) unsigned char smem[];
   SolidSums *lut = reinterpret_cast<SolidSums *>(smem);
   const int warps = blockDim.x / kLanes;
   Edge *edges = reinterpret_cast<Edge *>(smem + 512 * sizeof(SolidSums));
@@ -142,7 +144,6 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   const int lane = threadIdx.x & (kLanes - 1), w = threadIdx.x / kLanes;
 
   // The region: its first column and row, and the outputs it owns.
-  const int bx = blockIdx.x, by = blockIdx.y;
   const int nx = static_cast<int>(a.nx), ny = static_cast<int>(a.ny);
   const int64_t pitch = a.pitch;
   const int x0 = bx * g.ox - g.lead_x, y0 = by * g.oy - g.lead_y;
@@ -504,50 +505,110 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
 }
 
 template <typename T, int kR, bool kSr>
-cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
-                              int nsteps, cudaStream_t s) {
-  auto kern = lbm_resident_kernel<T, kR, kSr>;
+__global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
+    lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  resident_region<T, kR, kSr>(a, g, blockIdx.x, blockIdx.y, nsteps, smem);
+}
+
+// A batch's regions: one block per region of the work list.  The launch state
+// stays in shared memory, read where the region needs it.
+template <typename T, int kR, bool kSr>
+__global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
+    lbm_resident_batch_kernel(const ResidentBatch b, int nsteps) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(16) unsigned char raw_a[sizeof(StepLaunch)];
+  __shared__ __align__(16) unsigned char raw_g[sizeof(ResidentTiles)];
+  StepLaunch &a = *reinterpret_cast<StepLaunch *>(raw_a);
+  ResidentTiles &g = *reinterpret_cast<ResidentTiles *>(raw_g);
+  const int4 item = b.items[blockIdx.x];  // member, region x, region y
+  if (threadIdx.x == 0) {
+    const BatchMember &m = b.members[item.x];
+    fill_launch(a, m, (m.cur ^ b.parity) & 1, b.storage, b.clock);
+    g = m.tiles;
+  }
+  __syncthreads();
+  resident_region<T, kR, kSr>(a, g, item.y, item.z, nsteps, smem);
+  // the clock of the launches that follow
+  if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
+}
+
+// Launches a region kernel, to start while the launch before it ends.
+template <auto kKern, typename... A>
+cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
+                           cudaStream_t s, const A &...args) {
   static cudaError_t attr = cudaFuncSetAttribute(
-      kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      resident_smem<kR>(kResMaxWarps));
+      kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);
   if (attr != cudaSuccess) return attr;
   (void)cudaGetLastError();
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.gx, g.gy);
-  cfg.blockDim = dim3(g.warps * kLanes);
-  cfg.dynamicSmemBytes = resident_smem<kR>(g.warps);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(warps * kLanes);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a, g, nsteps);
+  return cudaLaunchKernelEx(&cfg, kKern, args...);
+}
+
+template <typename T, int kR, bool kSr>
+cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
+                              int nsteps, cudaStream_t s) {
+  return launch_regions<lbm_resident_kernel<T, kR, kSr>>(
+      dim3(g.gx, g.gy), g.warps, resident_smem<kR>(g.warps),
+      resident_smem<kR>(kResMaxWarps), s, a, g, nsteps);
+}
+
+template <typename T, int kR, bool kSr>
+cudaError_t launch_resident_batch_k(const ResidentBatch &b, int nsteps,
+                                    cudaStream_t s) {
+  return launch_regions<lbm_resident_batch_kernel<T, kR, kSr>>(
+      dim3(static_cast<unsigned>(b.nitems)), b.warps,
+      resident_smem<kR>(b.warps), resident_smem<kR>(kResMaxWarps), s, b,
+      nsteps);
+}
+
+// f(rows per warp, stochastic rounding) as compile-time constants
+template <typename F>
+cudaError_t with_rows(int rows, bool sr, F &&f) {
+  auto go = [&](auto r) {
+    return sr ? f(r, std::true_type{}) : f(r, std::false_type{});
+  };
+  switch (rows) {
+    case 2: return go(std::integral_constant<int, 2>{});
+    case 4: return go(std::integral_constant<int, 4>{});
+    default: return go(std::integral_constant<int, 8>{});
+  }
 }
 
 template <typename T>
 cudaError_t launch_resident_t(const StepLaunch &a, const ResidentTiles &g,
                               int nsteps, cudaStream_t s) {
-  if (a.sr) {
-    switch (g.rows) {
-      case 2: return launch_resident_k<T, 2, true>(a, g, nsteps, s);
-      case 4: return launch_resident_k<T, 4, true>(a, g, nsteps, s);
-      default: return launch_resident_k<T, 8, true>(a, g, nsteps, s);
-    }
-  }
-  switch (g.rows) {
-    case 2: return launch_resident_k<T, 2, false>(a, g, nsteps, s);
-    case 4: return launch_resident_k<T, 4, false>(a, g, nsteps, s);
-    default: return launch_resident_k<T, 8, false>(a, g, nsteps, s);
-  }
+  return with_rows(g.rows, a.sr != 0, [&](auto r, auto sr) {
+    return launch_resident_k<T, decltype(r)::value, decltype(sr)::value>(
+        a, g, nsteps, s);
+  });
+}
+
+template <typename T>
+cudaError_t launch_resident_batch_t(const ResidentBatch &b, int nsteps,
+                                    cudaStream_t s) {
+  return with_rows(b.rows, b.sr != 0, [&](auto r, auto sr) {
+    return launch_resident_batch_k<T, decltype(r)::value,
+                                   decltype(sr)::value>(b, nsteps, s);
+  });
 }
 
 // The launchers of storage type T, as the table lbm_step.cu dispatches on.
 template <typename T>
 constexpr StorageOps make_ops() {
   return StorageOps{&launch_step_t<T>, &launch_batch_t<T>, &choose_variant_t<T>,
-                    &launch_resident_t<T>, &pack_t<T>,     &unpack_t<T>,
-                    &solid_t<T>,       &change_t<T>};
+                    &launch_resident_t<T>, &launch_resident_batch_t<T>,
+                    &pack_t<T>,        &unpack_t<T>,       &solid_t<T>,
+                    &change_t<T>};
 }
 
 }  // namespace

@@ -214,11 +214,10 @@ cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s) {
   return ops(a.storage).step(a, reduce, s);
 }
 
-// Tiling with `rows` rows per warp, `warps` warps and `steps` steps a launch.
-static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
-                                    int periodic_y, int rows, int warps,
-                                    int steps) {
+ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
+                             int steps) {
   constexpr int kWidth = 64;
+  const int64_t nx = d.nx, ny = d.ny;
   ResidentTiles g;
   const int height = rows * warps;
   g.rows = rows;
@@ -228,7 +227,7 @@ static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
   g.hy = steps;
   g.ox = kWidth - 2 * g.hx;
   g.oy = height - 2 * g.hy;
-  if (!periodic_x) {
+  if (!d.periodic_x) {
     // one lane of outside columns before the domain, one column after it
     g.lead_x = 2;
     if (nx <= kWidth - 3) {
@@ -241,7 +240,7 @@ static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
     g.lead_x = g.hx;
     g.gx = static_cast<int>((nx + g.ox - 1) / g.ox);
   }
-  if (!periodic_y) {
+  if (!d.periodic_y) {
     if (ny <= height) {
       g.hy = 0;
       g.gy = 1;
@@ -256,13 +255,14 @@ static ResidentTiles resident_tiles(int64_t nx, int64_t ny, int periodic_x,
   return g;
 }
 
-ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
-                              int periodic_y, int nsteps) {
+ResidentTiles choose_resident(const ResidentShape *shapes, int count,
+                              int nsteps) {
   ResidentTiles best;
-  // rows wrap at most once, and a region's offsets fit 32 bits
-  if (nx < 8 || ny < 8 || nx > (1 << 23) || nsteps < 1 ||
-      forced_variant() >= 0)
-    return best;
+  if (count < 1 || nsteps < 1 || forced_variant() >= 0) return best;
+  for (int i = 0; i < count; ++i)  // rows wrap at most once, and a region's
+    if (shapes[i].nx < 8 || shapes[i].ny < 8 ||  // offsets fit 32 bits
+        shapes[i].nx > (1 << 23))
+      return best;
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -285,14 +285,21 @@ ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
   // shares, so that domains of many regions want short ones (3 or 4 steps on
   // 64 x 64 regions from about 1500^2 on).  Fitted to launches on a GB300
   // (64^2 .. 8192^2 boxes).
+  // Many domains try fewer tilings: the search is a few hundred thousand
+  // region counts at most.
   double best_us = 0.0;
   for (int r = 2; r <= 8; r *= 2)
     for (int w = 1; w <= kWarpsPerSm; ++w)
       for (int t = 1; t <= nsteps; ++t) {
-        const ResidentTiles g =
-            resident_tiles(nx, ny, periodic_x, periodic_y, r, w, t);
+        if (count > 1 && (w % 4 || t > 8)) continue;
+        ResidentTiles g;
+        int64_t blocks = 0;
+        for (int i = 0; i < count; ++i) {
+          g = resident_tiles(shapes[i], r, w, t);
+          if (g.rows == 0) break;
+          blocks += static_cast<int64_t>(g.gx) * g.gy;
+        }
         if (g.rows == 0) continue;
-        const int64_t blocks = static_cast<int64_t>(g.gx) * g.gy;
         const int64_t per_sm = (blocks + sms - 1) / sms;
         const int c = kWarpsPerSm / w;
         // k blocks on an SM at a time (four schedulers: warps count by
@@ -301,7 +308,9 @@ ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
         auto round_us = [&](int64_t k) {
           const int rows = static_cast<int>(k) * r * ((w + 3) / 4 * 4);
           const double steps = t * step_us(r, rows);
-          const double over = 1.3 + 0.02 * rows;
+          // (a batch's blocks fetch their member first, and more of them
+          // touch an edge)
+          const double over = (count > 1 ? 2.3 : 1.3) + 0.02 * rows;
           return steps + (per_sm > k && k > 1
                               ? fmax(0.25 * over, over - 0.42 * steps) : over);
         };
@@ -319,6 +328,11 @@ ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
 cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
                             int nsteps, cudaStream_t s) {
   return ops(a.storage).resident(a, g, nsteps, s);
+}
+
+cudaError_t launch_resident_batch(const ResidentBatch &b, int nsteps,
+                                  cudaStream_t s) {
+  return ops(b.storage).resident_batch(b, nsteps, s);
 }
 
 cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,

@@ -49,6 +49,18 @@ struct StepLaunch {
   float g_sc = 0.0f;
 };
 
+// Tiling of a launch that takes several steps on register-resident regions
+// of 64 columns x (rows * warps) rows (lbm_resident.cuh): region (bx, by)
+// starts at column bx * ox - lead_x and row by * oy - lead_y and owns the
+// nodes at least (hx, hy) inside its sides that face other regions.
+struct ResidentTiles {
+  int rows = 0;    // rows per warp (2, 4 or 8); 0: no such launch
+  int warps = 0;   // warps per block (stacked in y)
+  int steps = 0;   // steps a launch may take
+  int gx = 0, gy = 0;
+  int ox = 0, oy = 0, hx = 0, hy = 0, lead_x = 0, lead_y = 0;
+};
+
 // One member of a batch (see launch_batch): both field copies, the copy that
 // holds its current state, its node types and problem data, and its own
 // reduction partials and result slot.
@@ -67,6 +79,7 @@ struct BatchMember {
   int sr;            // stochastic rounding (as StepLaunch::sr)
   int64_t step_base; // member's step count minus the batch clock
   const uint8_t *clean;  // clean-tile flags for the batch's variant
+  ResidentTiles tiles;   // tiling of the batch's multi-step launches
 };
 
 struct BatchLaunch {
@@ -80,16 +93,18 @@ struct BatchLaunch {
   unsigned int *done;     // blocks finished in this launch (zero between)
 };
 
-// Tiling of a launch that takes several steps on register-resident regions
-// of 64 columns x (rows * warps) rows (lbm_resident.cuh): region (bx, by)
-// starts at column bx * ox - lead_x and row by * oy - lead_y and owns the
-// nodes at least (hx, hy) inside its sides that face other regions.
-struct ResidentTiles {
-  int rows = 0;    // rows per warp (2, 4 or 8); 0: no such launch
-  int warps = 0;   // warps per block (stacked in y)
-  int steps = 0;   // steps a launch may take
-  int gx = 0, gy = 0;
-  int ox = 0, oy = 0, hx = 0, hy = 0, lead_x = 0, lead_y = 0;
+// A launch that takes several steps on the regions of many members, which
+// share `rows`, `warps` and the rounding mode.
+struct ResidentBatch {
+  const BatchMember *members;
+  const int4 *items;    // (member, region x, region y, -)
+  int nitems;
+  int rows, warps;
+  int sr;               // stochastic rounding, the same for every item
+  int storage;
+  int parity;           // launches taken within the call, mod 2
+  unsigned clock;       // batch clock before the launch
+  unsigned *next_clock; // receives the clock after it
 };
 
 // The launchers of one storage format.  The kernels are templates on the
@@ -103,6 +118,8 @@ struct StorageOps {
   int (*choose)(int64_t nx, int64_t ny);
   cudaError_t (*resident)(const StepLaunch &a, const ResidentTiles &g,
                           int nsteps, cudaStream_t s);
+  cudaError_t (*resident_batch)(const ResidentBatch &b, int nsteps,
+                                cudaStream_t s);
   cudaError_t (*pack)(const double *staging, Fields f, int64_t nx,
                       int64_t pitch, int64_t y0, int64_t rows,
                       cudaStream_t s);
@@ -167,14 +184,24 @@ cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,
 // (sum |du|^2, sum |u|^2, sum (rho - 1)) and raises the flag on instability.
 cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s);
 
-// Tiling for a run of nsteps steps on an nx x ny domain (rows = 0: none; the
-// steps are then launched one by one).
-ResidentTiles choose_resident(int64_t nx, int64_t ny, int periodic_x,
-                              int periodic_y, int nsteps);
+// Tiling for runs of nsteps steps on one domain, or on several that share a
+// launch: rows, warps and steps in the result; rows = 0: none, the steps are
+// then launched one by one.
+struct ResidentShape {
+  int64_t nx, ny;
+  int periodic_x, periodic_y;
+};
+ResidentTiles choose_resident(const ResidentShape *shapes, int count,
+                              int nsteps);
+// The regions of one domain for the chosen rows, warps and steps.
+ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
+                             int steps);
 
 // Enqueues nsteps <= g.steps unreduced steps from a.src to a.dst.
 cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
                             int nsteps, cudaStream_t s);
+cudaError_t launch_resident_batch(const ResidentBatch &b, int nsteps,
+                                  cudaStream_t s);
 
 // Sums the partial triples of `nblocks` block tiles (kTileWarps each, added
 // in warp order per block) in FP64 in a fixed order into out[0..2].

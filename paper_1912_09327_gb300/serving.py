@@ -2,8 +2,8 @@
 
 Requests (a domain to solve to a steady-state residual) arrive over time.
 The service keeps every admitted domain's fields on the device and advances
-all of them together with the batched step (one launch per time step for the
-whole batch, lbm_batch_step).  Between chunks of steps it reads every member's
+all of them together with the batched step (launches shared by the whole
+batch, lbm_batch_step).  Between chunks of steps it reads every member's
 residual with one copy, retires the converged members (their final state is
 downloaded and their memory freed), and admits waiting requests while batch
 slots, the device-memory budget and the active-node budget allow: new work

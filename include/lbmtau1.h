@@ -170,7 +170,8 @@ int lbm_set_moments(lbm_ctx *ctx, const double *rho, const double *jx,
  * returns and checks for rho <= 0 or non-finite values.  nsteps = 0 is a
  * no-op.  The steps before the last are taken several per launch, unless a
  * tile variant was set (lbm_set_variant), a side is shorter than 8 nodes or
- * the step is the multiphase one: those take one launch per step, and on a
+ * longer than 2^23 along x, or a multiphase step rounds stochastically: those
+ * take one launch per step, and on a
  * stream that can be captured (not the legacy default stream, and not under a
  * capture of the caller's) runs of 16 inner steps are then replayed from a
  * CUDA graph captured at first use (FP32 storage, or 16-bit storage rounded

@@ -437,13 +437,14 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   // unless the caller chose a tile variant of the single-step kernel.  Two
   // inner steps at least: a launch for one costs what the kernel it replaces
   // costs.
-  if (nsteps >= 3 && !c->variant_set && c->p.sc_g == 0.0) {
+  const bool sc = c->p.sc_g != 0.0;
+  if (nsteps >= 3 && !c->variant_set && !(sc && a.sr)) {
     int64_t left = nsteps - 1;
     const int run = static_cast<int>(left < lbmtau1::kLongRun
                                          ? left : lbmtau1::kLongRun);
     if (!c->tiles_known[run]) {
       const lbmtau1::ResidentShape d = {c->p.nx, c->p.ny, a.periodic_x,
-                                        a.periodic_y};
+                                        a.periodic_y, sc ? 2 : 1};
       c->tiles[run] = lbmtau1::choose_resident(&d, 1, run);
       c->tiles_known[run] = true;
     }

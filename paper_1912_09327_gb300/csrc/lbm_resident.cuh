@@ -23,6 +23,13 @@
 // issue slots, and their code instruction fetches: 1.07 no-instruction stalls
 // per issue before, 0.24 after).
 //
+// The multiphase step runs here too, in two passes a step with a barrier each:
+// the potentials and their horizontal terms give every row its force, which is
+// added to the momentum in its registers; then the single-phase step.  Its
+// result reaches two nodes to each side, so a region's rim goes stale by two
+// nodes a step (drop 2048^2: 61.8 us a step launched one by one, 21.1 here in
+// launches of two).
+//
 // Every node's arithmetic is that of step_tile (lbm_kernels.cuh), operation by
 // operation, and 16-bit formats round to storage after every step with the
 // random bits of the node's own place: the states are equal bit for bit.
@@ -57,10 +64,18 @@ struct Edge {
   float2 zy[kLanes];
 };
 
-template <int kR>
+// The multiphase step's boundary rows: their potential and its horizontal
+// difference and sum.
+struct PsiEdge {
+  float2 c[kLanes], a[kLanes], s[kLanes];
+};
+static_assert(sizeof(PsiEdge) <= sizeof(Edge), "shares the edges' buffer");
+
+template <int kR, bool kSC>
 __host__ __device__ constexpr int resident_smem(int warps) {
   return 512 * static_cast<int>(sizeof(SolidSums)) +
-         warps * (4 * static_cast<int>(sizeof(Edge)) + kR * kLanes * 4);
+         warps * (4 * static_cast<int>(sizeof(Edge)) +
+                  kR * kLanes * (kSC ? 4 + 16 : 4));
 }
 
 // Programmatic dependent launch: wait until the launches before this one
@@ -129,8 +144,8 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
   }
 }
 
-// Takes nsteps steps on region (bx, by); every thread of the block calls it.
-template <typename T, int kR, bool kSr>
+// Takes nsteps steps on region (bx, by) (kSC: Shan-Chen multiphase steps); every thread of the block calls it.
+template <typename T, int kR, bool kSr, bool kSC>
 __device__ __forceinline__ void resident_region(const StepLaunch &a,
                                                 const ResidentTiles &g, int bx,
                                                 int by, int nsteps,
@@ -141,6 +156,9 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   const int warps = blockDim.x / kLanes;
   Edge *edges = reinterpret_cast<Edge *>(smem + 512 * sizeof(SolidSums));
   unsigned *codes = reinterpret_cast<unsigned *>(edges + 4 * warps);
+  // kSC: the momentum of kept nodes, which the force does not change (a
+  // node's register holds its momentum with the force while a step goes on)
+  float4 *kept = reinterpret_cast<float4 *>(codes + warps * kR * kLanes);
   const int lane = threadIdx.x & (kLanes - 1), w = threadIdx.x / kLanes;
 
   // The region: its first column and row, and the outputs it owns.
@@ -293,6 +311,9 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
       // a solid node's momentum as a source: -F (zero momentum j + F)
       if (own & 2u) { d[r].x = 0.f; zx[r].x = -fx; zy[r].x = -fy; }
       if (own & 4u) { d[r].y = 0.f; zx[r].y = -fx; zy[r].y = -fy; }
+      if constexpr (kSC)
+        kept[(w * kR + r) * kLanes + lane] =
+            make_float4(zx[r].x, zx[r].y, zy[r].x, zy[r].y);
       lo = own;
       own = hi;
       fc = fn;
@@ -318,7 +339,63 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
     for (int t = 0; t < nsteps; ++t) {
       const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
       const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
-      Edge *mine = edges + ((t & 1) * warps + w) * 2;  // [0] down, [1] up
+      // [0] down, [1] up (kSC: two barriers a step, so one buffer; the other
+      // holds the potentials)
+      Edge *mine = edges + ((kSC ? 0 : t & 1) * warps + w) * 2;
+      if constexpr (kSC) {
+        // The force of every row (Eq. f_sc; the terms and their order are
+        // step_tile's), added to its momentum.
+        struct Psi {
+          float2 c, a, s;
+        };
+        const float2 mg = bc(-a.g_sc), one = bc(1.0f);
+        const float2 w1_9 = bc(k1_9), w1_36 = bc(k1_36);
+        auto terms = [&](int r) -> Psi {
+          const float2 rho = add(d[r], one);
+          float2 c = make_float2(1.0f - __expf(-rho.x), 1.0f - __expf(-rho.y));
+          if (kWalls && ((walls >> r) & 1u)) {
+            const unsigned code = codes[(w * kR + r) * kLanes + lane];
+            if (code & (1u << 4)) c.x = 0.f;   // the node's own solid bit
+            if (code & (1u << 13)) c.y = 0.f;
+          }
+          const float l = __shfl_up_sync(kFull, c.y, 1);
+          const float p = __shfl_down_sync(kFull, c.x, 1);
+          return {c, make_float2(__fsub_rn(c.y, l), __fsub_rn(p, c.x)),
+                  make_float2(__fadd_rn(c.y, l), __fadd_rn(p, c.x))};
+        };
+        auto force = [&](int r, const Psi &lo, const Psi &own, const Psi &hi) {
+          const float2 k = mul(own.c, mg);
+          const float2 sx = fma2(w1_36, add(lo.a, hi.a), mul(w1_9, own.a));
+          const float2 sy =
+              fma2(w1_9, sub(hi.c, lo.c), mul(w1_36, sub(hi.s, lo.s)));
+          zx[r] = add(zx[r], mul(k, sx));
+          zy[r] = add(zy[r], mul(k, sy));
+        };
+        PsiEdge *psi = reinterpret_cast<PsiEdge *>(edges + 2 * warps) + 2 * w;
+        Psi lo, own, r0, r1;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+          const Psi now = terms(r);
+          if (r == 0 || r == kR - 1) {
+            PsiEdge &e = psi[r == 0 ? 0 : 1];
+            e.c[lane] = now.c;
+            e.a[lane] = now.a;
+            e.s[lane] = now.s;
+          }
+          if (r == 0) r0 = now;
+          if (r == 1) r1 = now;
+          if (r > 1) force(r - 1, lo, own, now);
+          if (r > 0) lo = own;
+          own = now;
+        }
+        __syncthreads();
+        auto edge = [&](bool there, const PsiEdge *e) -> Psi {
+          if (!there) return {bc(0.f), bc(0.f), bc(0.f)};
+          return {e->c[lane], e->a[lane], e->s[lane]};
+        };
+        force(0, edge(w > 0, psi - 1), r0, r1);
+        force(kR - 1, lo, own, edge(w + 1 < warps, psi + 2));
+      }
 
       // completes row r: acc holds South(r - 1) + Same(r) with the vertical
       // difference to row r - 1, (nd, nx_, ny_) the row above's contribution
@@ -357,9 +434,15 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         }
         if (kWalls && ((keep >> r) & 1u)) {
           const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
+          float2 xk = zxO, yk = zyO;
+          if constexpr (kSC) {
+            const float4 k = kept[(w * kR + r) * kLanes + lane];
+            xk = make_float2(k.x, k.y);
+            yk = make_float2(k.z, k.w);
+          }
           dn = make_float2(f0 ? dn.x : dO.x, f1 ? dn.y : dO.y);
-          xn = make_float2(f0 ? xn.x : zxO.x, f1 ? xn.y : zxO.y);
-          yn = make_float2(f0 ? yn.x : zyO.x, f1 ? yn.y : zyO.y);
+          xn = make_float2(f0 ? xn.x : xk.x, f1 ? xn.y : xk.y);
+          yn = make_float2(f0 ? yn.x : yk.x, f1 ? yn.y : yk.y);
         }
         d[r] = dn;
         zx[r] = xn;
@@ -504,11 +587,11 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   }
 }
 
-template <typename T, int kR, bool kSr>
+template <typename T, int kR, bool kSr, bool kSC>
 __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
   extern __shared__ __align__(128) unsigned char smem[];
-  resident_region<T, kR, kSr>(a, g, blockIdx.x, blockIdx.y, nsteps, smem);
+  resident_region<T, kR, kSr, kSC>(a, g, blockIdx.x, blockIdx.y, nsteps, smem);
 }
 
 // A batch's regions: one block per region of the work list.  The launch state
@@ -528,7 +611,7 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     g = m.tiles;
   }
   __syncthreads();
-  resident_region<T, kR, kSr>(a, g, item.y, item.z, nsteps, smem);
+  resident_region<T, kR, kSr, false>(a, g, item.y, item.z, nsteps, smem);
   // the clock of the launches that follow
   if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
 }
@@ -554,12 +637,12 @@ cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
   return cudaLaunchKernelEx(&cfg, kKern, args...);
 }
 
-template <typename T, int kR, bool kSr>
+template <typename T, int kR, bool kSr, bool kSC>
 cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
                               int nsteps, cudaStream_t s) {
-  return launch_regions<lbm_resident_kernel<T, kR, kSr>>(
-      dim3(g.gx, g.gy), g.warps, resident_smem<kR>(g.warps),
-      resident_smem<kR>(kResMaxWarps), s, a, g, nsteps);
+  return launch_regions<lbm_resident_kernel<T, kR, kSr, kSC>>(
+      dim3(g.gx, g.gy), g.warps, resident_smem<kR, kSC>(g.warps),
+      resident_smem<kR, kSC>(kResMaxWarps), s, a, g, nsteps);
 }
 
 template <typename T, int kR, bool kSr>
@@ -567,7 +650,7 @@ cudaError_t launch_resident_batch_k(const ResidentBatch &b, int nsteps,
                                     cudaStream_t s) {
   return launch_regions<lbm_resident_batch_kernel<T, kR, kSr>>(
       dim3(static_cast<unsigned>(b.nitems)), b.warps,
-      resident_smem<kR>(b.warps), resident_smem<kR>(kResMaxWarps), s, b,
+      resident_smem<kR, false>(b.warps), resident_smem<kR, false>(kResMaxWarps), s, b,
       nsteps);
 }
 
@@ -587,9 +670,17 @@ cudaError_t with_rows(int rows, bool sr, F &&f) {
 template <typename T>
 cudaError_t launch_resident_t(const StepLaunch &a, const ResidentTiles &g,
                               int nsteps, cudaStream_t s) {
+  if (a.g_sc != 0.0f) {
+    if constexpr (std::is_same<T, float>::value)
+      return with_rows(g.rows, false, [&](auto r, auto) {
+        return launch_resident_k<T, decltype(r)::value, false, true>(
+            a, g, nsteps, s);
+      });
+    return cudaErrorInvalidValue;
+  }
   return with_rows(g.rows, a.sr != 0, [&](auto r, auto sr) {
-    return launch_resident_k<T, decltype(r)::value, decltype(sr)::value>(
-        a, g, nsteps, s);
+    return launch_resident_k<T, decltype(r)::value, decltype(sr)::value,
+                             false>(a, g, nsteps, s);
   });
 }
 

@@ -223,8 +223,8 @@ ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
   g.rows = rows;
   g.warps = warps;
   g.steps = steps;
-  g.hx = (steps + 1) & ~1;
-  g.hy = steps;
+  g.hx = (d.reach * steps + 1) & ~1;
+  g.hy = d.reach * steps;
   g.ox = kWidth - 2 * g.hx;
   g.oy = height - 2 * g.hy;
   if (!d.periodic_x) {
@@ -273,11 +273,13 @@ ResidentTiles choose_resident(const ResidentShape *shapes, int count,
   }();
   if (sms <= 0) return best;
   constexpr int kWarpsPerSm = 16;
+  // (the multiphase step takes 1.6 times as long)
+  const double slow = shapes[0].reach > 1 ? 1.6 : 1.0;
   // time of one step on an SM whose resident warps hold `rows` rows of 64
   // columns: 3400 nodes/us once 16 warps are there, and at least the chain
   // of a warp's own r rows
-  auto step_us = [](int r, int rows) {
-    return fmax(0.0188 * rows + 0.1, 0.18 + 0.1 * r);
+  auto step_us = [slow](int r, int rows) {
+    return slow * fmax(0.0188 * rows + 0.1, 0.18 + 0.1 * r);
   };
   // The tiling with the shortest expected time per step.  A launch of t steps
   // pays for its loads and stores once, so that small domains want long

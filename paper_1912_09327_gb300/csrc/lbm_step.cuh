@@ -190,6 +190,8 @@ cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s);
 struct ResidentShape {
   int64_t nx, ny;
   int periodic_x, periodic_y;
+  int reach = 1;  // nodes a step's result depends on to each side (2: the
+                  // multiphase step, whose sources see their neighbours)
 };
 ResidentTiles choose_resident(const ResidentShape *shapes, int count,
                               int nsteps);

@@ -57,6 +57,25 @@ def test_equals_one_launch_per_step(b, nx, ny, storage, rounding):
         assert abs(got[1] - want[1]) <= 1.5e-5 * 0.1 * nx * ny
 
 
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_multiphase_equals_one_launch_per_step(b, nx, ny):
+    """The multiphase step, whose rim goes stale by two nodes a step: random
+    densities with walls and fixed nodes in every periodicity, bit for bit."""
+    for k, per in enumerate([(False, False), (True, False), (False, True),
+                             (True, True)]):
+        p = wl.multiphase_random(nx, ny, seed=7 * nx + ny + k, periodic=per)
+        got = []
+        for variant in (-1, 3):
+            d = b.Domain.from_problem(p)
+            d.set_variant(variant)
+            for n in (3, 12, 4 + k):
+                d.step(n)
+            got.append(d.get_state())
+            d.close()
+        for x, y in zip(*got):
+            assert np.array_equal(x.view(np.uint32), y.view(np.uint32)), per
+
+
 def test_captured_calls_replay(b):
     """A caller's graph of an even number of steps leaves the state in the
     copy it found it in, so that replays go on from one another."""

@@ -203,7 +203,9 @@ int32_t lbm_variant(lbm_ctx *ctx);
  * On expiry the warp stops, lets its copies still in flight land (that drain
  * keeps the one-second bound whatever the limit) and raises a flag, which
  * lbm_residual reports as LBM_E_CUDA; the fields are then incomplete, and
- * loading a state (lbm_set_moments / lbm_set_state) clears the flag.  A limit
+ * loading a state (lbm_set_moments / lbm_set_state) clears the flag.  A call's
+ * reduced last step goes through the step kernel whenever the limit is not
+ * the default (else it may run on regions that stage nothing).  A limit
  * of 0 makes every such wait give up at once without looking, which tests
  * this path without any fault.  Errors: LBM_E_INVAL (ns < 0 or > 10^9).
  */

@@ -22,6 +22,7 @@ namespace {
 constexpr int64_t kPitchAlign = 32;           // nodes; rows start 128-B aligned
 constexpr size_t kAlign = 256;                // bytes; every workspace region
 constexpr int64_t kStagingNodes = 1 << 20;    // host-transfer chunk (nodes)
+constexpr unsigned long long kDefaultWaitNs = 1000000000ull;
 constexpr int64_t kMaxExtent = (int64_t(1) << 30) - 1;  // rows index in 32 bits
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -163,12 +164,13 @@ int lbm_create(const lbm_params *p, void *dev_workspace, size_t workspace_bytes,
   c->variant = -1;
   c->variant_set = false;
   for (bool &k : c->tiles_known) k = false;
+  c->reduce_known = false;
   c->steps = 0;
   c->graph[0] = c->graph[1] = nullptr;
   c->graph_variant[0] = c->graph_variant[1] = -1;
   c->graphs_off = cuda_stream == nullptr || c->stream == cudaStreamLegacy ||
                   c->stream == cudaStreamPerThread;
-  c->wait_ns = 1000000000ull;
+  c->wait_ns = kDefaultWaitNs;
   c->has_geometry = false;
   c->has_residual = false;
   c->n_fluid = 0;
@@ -212,6 +214,7 @@ int lbm_set_geometry(lbm_ctx *c, const uint8_t *host_mask) {
   c->cur = 0;
   c->n_fluid = fluid;
   c->clean_variant = -1;  // new node types: flags computed again
+  c->reduce_known = false;
   c->has_geometry = true;
   c->err[0] = '\0';
   return LBM_OK;
@@ -335,6 +338,28 @@ int select_variant(lbm_ctx *c) {
   return LBM_OK;
 }
 
+// Chooses how the context takes a call's reduced last step (reduce_tiles).  A
+// single step on regions beats the single-step kernel on small and middling
+// domains (1024^2 27 -> 19 us with the finalize, 64^2 25 -> 12); where most
+// tiles of a large domain are clean, that kernel's long march with its copies
+// in flight is the faster way to move 24 bytes a node (8192^2 379 against
+// 543 us).
+int choose_reduce(lbm_ctx *c, const lbmtau1::ResidentShape &dom) {
+  c->reduce_tiles = lbmtau1::ResidentTiles();
+  c->reduce_known = true;
+  const int v = lbmtau1::choose_variant(c->p.nx, c->p.ny, c->p.storage);
+  if (lbmtau1::dual_variant(v, c->p.nx, c->p.ny) >= 0) {
+    if (c->variant < 0) {
+      const int st = select_variant(c);
+      if (st) return st;
+    }
+    if (lbmtau1::variant_has_clean_code(c->variant)) return LBM_OK;
+  }
+  c->reduce_tiles = lbmtau1::choose_resident(
+      &dom, 1, 1, c->L.nblocks * lbmtau1::kTileWarps);
+  return LBM_OK;
+}
+
 constexpr int64_t kGraphChunk = 16;  // steps per captured graph (even)
 
 // kGraphChunk unreduced steps from the current copy as one graph launch
@@ -412,19 +437,6 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   a.partials = c->partials;
   a.flag = c->flag;
   a.storage = c->p.storage;
-  if (c->variant < 0) {
-    const int st = select_variant(c);
-    if (st) return st;
-  }
-  a.variant = c->variant;
-  if (c->clean_variant != c->variant) {
-    cudaError_t e = lbmtau1::launch_tile_flags(c->variant, c->mask, c->p.nx,
-                                               c->p.ny, c->L.pitch, c->clean,
-                                               c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "tile flags kernel launch");
-    c->clean_variant = c->variant;
-  }
-  a.clean = c->clean;
   a.wait_ns = c->wait_ns;
   a.sr = lbmtau1::stochastic_rounding(c->p.storage, c->p.rounding);
   // Steps 1 .. nsteps - 2 go in captured graph chunks when the rounding
@@ -433,19 +445,18 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   // capture) and the reduced last step are launched directly.
   const bool graphs = !a.sr;
   int64_t s = 0;
+  int64_t partial_blocks = 0;
   // Several steps per launch up to the reduced last one (lbm_resident.cuh),
-  // unless the caller chose a tile variant of the single-step kernel.  Two
-  // inner steps at least: a launch for one costs what the kernel it replaces
-  // costs.
+  // unless the caller chose a tile variant of the single-step kernel.
   const bool sc = c->p.sc_g != 0.0;
-  if (nsteps >= 3 && !c->variant_set && !(sc && a.sr)) {
+  const lbmtau1::ResidentShape dom = {c->p.nx, c->p.ny, a.periodic_x,
+                                      a.periodic_y, sc ? 2 : 1};
+  if (nsteps >= 2 && !c->variant_set && !(sc && a.sr)) {
     int64_t left = nsteps - 1;
     const int run = static_cast<int>(left < lbmtau1::kLongRun
                                          ? left : lbmtau1::kLongRun);
     if (!c->tiles_known[run]) {
-      const lbmtau1::ResidentShape d = {c->p.nx, c->p.ny, a.periodic_x,
-                                        a.periodic_y, sc ? 2 : 1};
-      c->tiles[run] = lbmtau1::choose_resident(&d, 1, run);
+      c->tiles[run] = lbmtau1::choose_resident(&dom, 1, run, INT64_MAX);
       c->tiles_known[run] = true;
     }
     const lbmtau1::ResidentTiles &tiles = c->tiles[run];
@@ -461,12 +472,51 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
       a.src = c->f[c->cur];
       a.dst = c->f[1 - c->cur];
       a.step = static_cast<uint32_t>(c->steps + s);
-      cudaError_t e = lbmtau1::launch_resident(a, tiles, n, c->stream);
+      cudaError_t e = lbmtau1::launch_resident(a, tiles, n, false,
+                                               c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
       c->cur = 1 - c->cur;
       s += n;
       left -= n;
     }
+  }
+  // The reduced last step on regions too, one partial triple each; unless the
+  // caller bounds the waits for staged rows, which are the single-step
+  // kernel's.
+  if (s == nsteps - 1 && !c->variant_set && !sc &&
+      c->wait_ns == kDefaultWaitNs) {
+    if (!c->reduce_known) {
+      const int st = choose_reduce(c, dom);
+      if (st) return st;
+    }
+    const lbmtau1::ResidentTiles &g = c->reduce_tiles;
+    if (g.rows > 0) {
+      a.src = c->f[c->cur];
+      a.dst = c->f[1 - c->cur];
+      a.step = static_cast<uint32_t>(c->steps + s);
+      cudaError_t e = lbmtau1::launch_resident(a, g, 1, true, c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+      c->cur = 1 - c->cur;
+      ++s;
+      partial_blocks = (static_cast<int64_t>(g.gx) * g.gy +
+                        lbmtau1::kTileWarps - 1) / lbmtau1::kTileWarps;
+    }
+  }
+  if (s < nsteps) {  // what is left goes through the single-step kernel
+    if (c->variant < 0) {
+      const int st = select_variant(c);
+      if (st) return st;
+    }
+    a.variant = c->variant;
+    if (c->clean_variant != c->variant) {
+      cudaError_t e = lbmtau1::launch_tile_flags(c->variant, c->mask, c->p.nx,
+                                                 c->p.ny, c->L.pitch, c->clean,
+                                                 c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "tile flags kernel launch");
+      c->clean_variant = c->variant;
+    }
+    a.clean = c->clean;
+    partial_blocks = lbmtau1::launched_blocks(c->p.nx, c->p.ny, c->variant);
   }
   while (s < nsteps) {
     if (graphs && s >= 1 && nsteps - 1 - s >= kGraphChunk) {
@@ -483,9 +533,8 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
     c->cur = 1 - c->cur;
     ++s;
   }
-  cudaError_t e = lbmtau1::launch_finalize(
-      c->partials, lbmtau1::launched_blocks(c->p.nx, c->p.ny, c->variant),
-      c->result, c->stream);
+  cudaError_t e = lbmtau1::launch_finalize(c->partials, partial_blocks,
+                                           c->result, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel launch");
   c->has_residual = true;
   c->steps += nsteps;

@@ -142,26 +142,20 @@ int build_regions(lbm_batch *b, int run) {
   }
   b->regions_for = run;
   b->nregions[0] = b->nregions[1] = 0;
-  b->tiles = lbmtau1::choose_resident(shapes.data(), n, run);
+  const int64_t most = b->max_tiles * lbmtau1::kTileWarps;
+  b->tiles = lbmtau1::choose_resident(shapes.data(), n, run, most);
   if (b->tiles.rows == 0) return LBM_OK;
   b->h_regions.clear();
-  const size_t most =
-      static_cast<size_t>(b->max_tiles) * lbmtau1::kTileWarps;
   for (int sr = 0; sr < 2; ++sr)
     for (int i = 0; i < n; ++i) {
       BatchMember &m = b->h_members[i];
       if ((m.sr != 0) != (sr != 0)) continue;
       const lbmtau1::ResidentTiles g = lbmtau1::resident_tiles(
           shapes[i], b->tiles.rows, b->tiles.warps, b->tiles.steps);
-      const size_t count = static_cast<size_t>(g.gx) * g.gy;
-      if (b->h_regions.size() + count > most) {
-        b->tiles.rows = 0;
-        return LBM_OK;
-      }
       for (int y = 0; y < g.gy; ++y)
         for (int x = 0; x < g.gx; ++x)
           b->h_regions.push_back(make_int4(i, x, y, 0));
-      b->nregions[sr] += static_cast<int>(count);
+      b->nregions[sr] += g.gx * g.gy;
     }
   cudaError_t e = cudaMemcpyAsync(b->d_regions, b->h_regions.data(),
                                   sizeof(int4) * b->h_regions.size(),

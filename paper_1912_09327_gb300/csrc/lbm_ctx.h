@@ -54,6 +54,8 @@ struct lbm_ctx {
   // each chosen at first use (tiles_known)
   lbmtau1::ResidentTiles tiles[lbmtau1::kLongRun + 1];
   bool tiles_known[lbmtau1::kLongRun + 1];
+  lbmtau1::ResidentTiles reduce_tiles;  // of a call's reduced last step
+  bool reduce_known;
   int64_t steps;        // steps taken (seeds stochastic rounding)
   // 16 unreduced steps captured as one CUDA graph, one per starting copy
   // (rebuilt when the tile variant changes); none on an uncapturable stream

@@ -381,6 +381,15 @@ __device__ __forceinline__ bool mbar_wait(
   return true;
 }
 
+// Programmatic dependent launch: wait until the launches before this one
+// have completed; let the next one start its prologue.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void fence_async_shared() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

@@ -29,7 +29,7 @@ constexpr int64_t kNoAllocMaxBlocks = int64_t(1) << 16;
 constexpr int64_t kNoAllocPartials = kNoAllocMaxBlocks * lbmtau1::kTileWarps;
 constexpr int kMaxDevices = 64;
 
-// Per-warp-tile partial triples (6 MB), then one slot whose low 4 bytes
+// Per-warp-tile (or per-region) partial triples (6 MB), then one slot whose low 4 bytes
 // hold the flag.
 static __device__ __align__(256) double
     g_step_scratch[3 * kNoAllocPartials + 1];
@@ -66,7 +66,7 @@ extern "C" int lbm_step_noalloc(const float *drho_in, const float *jx_in,
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
     return LBM_E_CUDA;
   const int variant = lbmtau1::choose_variant(nx, ny, lbmtau1::kStorageF32);
-  const int64_t blocks = lbmtau1::launched_blocks(nx, ny, variant);
+  int64_t blocks = lbmtau1::launched_blocks(nx, ny, variant);
   if (blocks > kNoAllocMaxBlocks)
     return LBM_E_INVAL;  // domain larger than the static scratch serves
   // Set-up on the first call on each device: the device address of the
@@ -102,7 +102,18 @@ extern "C" int lbm_step_noalloc(const float *drho_in, const float *jx_in,
   a.partials = partials;
   a.flag = flag;
   a.variant = variant;
-  if (lbmtau1::launch_step(a, true, s) != cudaSuccess) return LBM_E_CUDA;
+  // as lbm_step takes its reduced last step
+  const lbmtau1::ResidentShape dom = {nx, ny, a.periodic_x, a.periodic_y};
+  const lbmtau1::ResidentTiles g = lbmtau1::choose_resident(
+      &dom, 1, 1, lbmtau1::step_blocks(nx, ny) * lbmtau1::kTileWarps);
+  const int64_t regions = static_cast<int64_t>(g.gx) * g.gy;
+  if (g.rows > 0 && regions <= kNoAllocPartials) {
+    blocks = (regions + lbmtau1::kTileWarps - 1) / lbmtau1::kTileWarps;
+    if (lbmtau1::launch_resident(a, g, 1, true, s) != cudaSuccess)
+      return LBM_E_CUDA;
+  } else if (lbmtau1::launch_step(a, true, s) != cudaSuccess) {
+    return LBM_E_CUDA;
+  }
   if (lbmtau1::launch_finalize(partials, blocks, dev_sums, s) != cudaSuccess)
     return LBM_E_CUDA;
   if (cudaMemcpyAsync(dev_flags, flag, sizeof(unsigned),

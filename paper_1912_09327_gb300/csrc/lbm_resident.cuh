@@ -30,6 +30,11 @@
 // nodes a step (drop 2048^2: 61.8 us a step launched one by one, 21.1 here in
 // launches of two).
 //
+// A call's reduced last step runs here as a launch of one step (us per
+// lbm_step(ctx, 1), single-step kernel -> this, with the finalize: 64^2
+// 24.7 -> 6.5, 1024^2 26.7 -> 14.1, 2048^2 59 -> 34, 4096^2 156 -> 113), except
+// where a large domain's tiles are mostly clean (choose_reduce).
+//
 // Every node's arithmetic is that of step_tile (lbm_kernels.cuh), operation by
 // operation, and 16-bit formats round to storage after every step with the
 // random bits of the node's own place: the states are equal bit for bit.
@@ -76,15 +81,6 @@ __host__ __device__ constexpr int resident_smem(int warps) {
   return 512 * static_cast<int>(sizeof(SolidSums)) +
          warps * (4 * static_cast<int>(sizeof(Edge)) +
                   kR * kLanes * (kSC ? 4 + 16 : 4));
-}
-
-// Programmatic dependent launch: wait until the launches before this one
-// have completed; let the next one start its prologue.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void pdl_release() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // 1 / x as __fdividef(1, x) rounds it, without the product by one.
@@ -144,8 +140,10 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
   }
 }
 
-// Takes nsteps steps on region (bx, by) (kSC: Shan-Chen multiphase steps); every thread of the block calls it.
-template <typename T, int kR, bool kSr, bool kSC>
+// Takes nsteps steps on region (bx, by) (kSC: Shan-Chen multiphase steps;
+// kReduce: one step, whose residual and mass terms become the region's partial
+// triple); every thread of the block calls it.
+template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
 __device__ __forceinline__ void resident_region(const StepLaunch &a,
                                                 const ResidentTiles &g, int bx,
                                                 int by, int nsteps,
@@ -333,6 +331,40 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
                wm1_6 = bc(-k1_6), half = bc(0.5f), mhalf = bc(-0.5f),
                quarter = bc(0.25f);
 
+  // The residual's and the mass's sums, as step_tile takes them: FP32 per lane
+  // (the mass compensated over the rows), FP64 from the warps' sums on.
+  float2 rs_num = bc(0.f), rs_den = bc(0.f);
+  float rs_mass = 0.f, rs_comp = 0.f, rmin = 1.0f;
+  const bool own_cols = xb >= xlo && xb < xhi;
+  auto add_terms = [&](float2 dO, float2 xO, float2 yO, float2 dn, float2 xn,
+                       float2 yn, bool v0, bool v1) {
+    const float2 rn = add(dn, bc(1.0f));
+    const float2 irn = make_float2(rcp(rn.x), rcp(rn.y));
+    const float2 irn2 = mul(irn, irn);
+    const float2 t = mul(sub(dO, dn), irn);
+    const float2 ex = fma2(xO, t, sub(xn, xO));
+    const float2 ey = fma2(yO, t, sub(yn, yO));
+    const float2 nn = fma2(ex, ex, mul(ey, ey));
+    const float2 dd = fma2(xn, xn, mul(yn, yn));
+    float m = 0.f;
+    if (v0) {
+      rs_num.x = fmaf(nn.x, irn2.x, rs_num.x);
+      rs_den.x = fmaf(dd.x, irn2.x, rs_den.x);
+      m += dn.x;
+      rmin = fminf(rmin, rn.x);
+    }
+    if (v1) {
+      rs_num.y = fmaf(nn.y, irn2.y, rs_num.y);
+      rs_den.y = fmaf(dd.y, irn2.y, rs_den.y);
+      m += dn.y;
+      rmin = fminf(rmin, rn.y);
+    }
+    const float y = __fsub_rn(m, rs_comp);
+    const float u = __fadd_rn(rs_mass, y);
+    rs_comp = __fsub_rn(__fsub_rn(u, rs_mass), y);
+    rs_mass = u;
+  };
+
   // kWalls: some row of the block has solid neighbours or kept nodes
   auto march = [&](auto with_walls) {
     constexpr bool kWalls = decltype(with_walls)::value;
@@ -423,6 +455,13 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
           incy = fma2(lead_pow2(zyO), dither, incy);
         }
         float2 xn = add(zxO, incx), yn = add(zyO, incy);
+        if constexpr (kReduce) {
+          const bool own = own_cols && yb + r >= ylo && yb + r < yhi;
+          const unsigned fluid =
+              kWalls && ((keep >> r) & 1u) ? code >> 18 : 3u;
+          add_terms(dO, zxO, zyO, dn, xn, yn, own && (fluid & 1u),
+                    own && (fluid & 2u) && xb + 1 < nx);
+        }
         if constexpr (!kF32) {
           int row = yb + r;
           if constexpr (kSr)
@@ -569,6 +608,53 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   else
     march(std::false_type{});
 
+  if constexpr (kReduce) {
+    const bool finite = isfinite(rs_num.x) && isfinite(rs_num.y) &&
+                        isfinite(rs_den.x) && isfinite(rs_den.y) &&
+                        isfinite(rs_mass) && isfinite(rs_comp);
+    if (__any_sync(kFull, !(rmin > 0.f) || !finite) && lane == 0)
+      atomicOr(a.flag, kFlagUnstable);
+    // The lanes' sums, as pairs of addends, to shared memory; one warp per sum
+    // adds each lane's over the warps in two-float arithmetic (exact to about
+    // 2^-46) and only then goes to FP64: the FP64 pipe takes 16 cycles or
+    // more per warp instruction, and a butterfly of three sums in every warp
+    // kept it busy for 2 us per region.
+    __syncthreads();  // the edges' buffer is free
+    float2 *terms = reinterpret_cast<float2 *>(edges);
+    const int n = warps * kLanes;
+    terms[threadIdx.x] = rs_num;
+    terms[n + threadIdx.x] = rs_den;
+    terms[2 * n + threadIdx.x] = make_float2(rs_mass, -rs_comp);
+    __syncthreads();
+    const int region = by * g.gx + bx, last = g.gx * g.gy - 1;
+    for (int k = w; k < 3; k += warps) {
+      float hi = 0.f, lo = 0.f;
+      for (int i = 0; i < warps; ++i) {
+        const float2 v = terms[k * n + i * kLanes + lane];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {  // hi + lo += v, the rounding kept
+          const float x = e ? v.y : v.x;
+          const float s = __fadd_rn(hi, x);
+          const float t = __fsub_rn(s, hi);
+          lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)),
+                                       __fsub_rn(x, t)));
+          hi = s;
+        }
+      }
+      double total = static_cast<double>(hi) + lo;
+#pragma unroll
+      for (int o = kLanes / 2; o > 0; o >>= 1)
+        total += __shfl_xor_sync(kFull, total, o);
+      if (lane == 0) {
+        a.partials[3 * static_cast<int64_t>(region) + k] = total;
+        // the finalize kernel takes triples by fours
+        if (region == last)
+          for (int i = last + 1; i % kTileWarps; ++i)
+            a.partials[3 * static_cast<int64_t>(i) + k] = 0.0;
+      }
+    }
+  }
+
   // the owned outputs
   if (xb < xlo || xb >= xhi) return;
   const int64_t first = static_cast<int64_t>(y0) * pitch + x0;
@@ -587,11 +673,12 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   }
 }
 
-template <typename T, int kR, bool kSr, bool kSC>
+template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
 __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
   extern __shared__ __align__(128) unsigned char smem[];
-  resident_region<T, kR, kSr, kSC>(a, g, blockIdx.x, blockIdx.y, nsteps, smem);
+  resident_region<T, kR, kSr, kSC, kReduce>(a, g, blockIdx.x, blockIdx.y,
+                                            nsteps, smem);
 }
 
 // A batch's regions: one block per region of the work list.  The launch state
@@ -611,7 +698,7 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     g = m.tiles;
   }
   __syncthreads();
-  resident_region<T, kR, kSr, false>(a, g, item.y, item.z, nsteps, smem);
+  resident_region<T, kR, kSr, false, false>(a, g, item.y, item.z, nsteps, smem);
   // the clock of the launches that follow
   if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
 }
@@ -637,10 +724,10 @@ cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
   return cudaLaunchKernelEx(&cfg, kKern, args...);
 }
 
-template <typename T, int kR, bool kSr, bool kSC>
+template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
 cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
                               int nsteps, cudaStream_t s) {
-  return launch_regions<lbm_resident_kernel<T, kR, kSr, kSC>>(
+  return launch_regions<lbm_resident_kernel<T, kR, kSr, kSC, kReduce>>(
       dim3(g.gx, g.gy), g.warps, resident_smem<kR, kSC>(g.warps),
       resident_smem<kR, kSC>(kResMaxWarps), s, a, g, nsteps);
 }
@@ -669,18 +756,23 @@ cudaError_t with_rows(int rows, bool sr, F &&f) {
 
 template <typename T>
 cudaError_t launch_resident_t(const StepLaunch &a, const ResidentTiles &g,
-                              int nsteps, cudaStream_t s) {
+                              int nsteps, bool reduce, cudaStream_t s) {
   if (a.g_sc != 0.0f) {
     if constexpr (std::is_same<T, float>::value)
-      return with_rows(g.rows, false, [&](auto r, auto) {
-        return launch_resident_k<T, decltype(r)::value, false, true>(
-            a, g, nsteps, s);
-      });
+      if (!reduce)
+        return with_rows(g.rows, false, [&](auto r, auto) {
+          return launch_resident_k<T, decltype(r)::value, false, true, false>(
+              a, g, nsteps, s);
+        });
     return cudaErrorInvalidValue;
   }
+  if (reduce && nsteps != 1) return cudaErrorInvalidValue;
   return with_rows(g.rows, a.sr != 0, [&](auto r, auto sr) {
-    return launch_resident_k<T, decltype(r)::value, decltype(sr)::value,
-                             false>(a, g, nsteps, s);
+    constexpr int kR = decltype(r)::value;
+    constexpr bool kSr = decltype(sr)::value;
+    return reduce
+               ? launch_resident_k<T, kR, kSr, false, true>(a, g, 1, s)
+               : launch_resident_k<T, kR, kSr, false, false>(a, g, nsteps, s);
   });
 }
 

@@ -75,13 +75,15 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x < 3) m.result[threadIdx.x] = buf[threadIdx.x][0];
 }
 
-constexpr int kFinalizeThreads = 1024;
-
+// kThreads 1024, or 128 for few block tiles: the tree over the threads is FP64
+// adds and barriers, which a small domain's step otherwise waits for.
+template <int kFinalizeThreads>
 __global__ void __launch_bounds__(kFinalizeThreads)
     finalize_kernel(const double *__restrict__ partials, int64_t nblocks,
                     double *__restrict__ out) {
   __shared__ double buf[3][kFinalizeThreads];
   double s[3] = {0.0, 0.0, 0.0};
+  pdl_wait();  // launched while the step that writes the partials ends
   for (int64_t b = threadIdx.x; b < nblocks; b += kFinalizeThreads) {
     // the block tile's kWarps triples: 12 contiguous doubles, 16-byte aligned
     const double2 *p = reinterpret_cast<const double2 *>(partials + 3 * kWarps * b);
@@ -256,7 +258,7 @@ ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
 }
 
 ResidentTiles choose_resident(const ResidentShape *shapes, int count,
-                              int nsteps) {
+                              int nsteps, int64_t most) {
   ResidentTiles best;
   if (count < 1 || nsteps < 1 || forced_variant() >= 0) return best;
   for (int i = 0; i < count; ++i)  // rows wrap at most once, and a region's
@@ -301,7 +303,7 @@ ResidentTiles choose_resident(const ResidentShape *shapes, int count,
           if (g.rows == 0) break;
           blocks += static_cast<int64_t>(g.gx) * g.gy;
         }
-        if (g.rows == 0) continue;
+        if (g.rows == 0 || blocks > most) continue;
         const int64_t per_sm = (blocks + sms - 1) / sms;
         const int c = kWarpsPerSm / w;
         // k blocks on an SM at a time (four schedulers: warps count by
@@ -328,8 +330,8 @@ ResidentTiles choose_resident(const ResidentShape *shapes, int count,
 }
 
 cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
-                            int nsteps, cudaStream_t s) {
-  return ops(a.storage).resident(a, g, nsteps, s);
+                            int nsteps, bool reduce, cudaStream_t s) {
+  return ops(a.storage).resident(a, g, nsteps, reduce, s);
 }
 
 cudaError_t launch_resident_batch(const ResidentBatch &b, int nsteps,
@@ -358,8 +360,20 @@ cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,
 cudaError_t launch_finalize(const double *partials, int64_t nblocks,
                             double *out, cudaStream_t s) {
   (void)cudaGetLastError();
-  finalize_kernel<<<1, kFinalizeThreads, 0, s>>>(partials, nblocks, out);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(nblocks <= 128 ? 128 : 1024);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return nblocks <= 128
+             ? cudaLaunchKernelEx(&cfg, finalize_kernel<128>, partials,
+                                  nblocks, out)
+             : cudaLaunchKernelEx(&cfg, finalize_kernel<1024>, partials,
+                                  nblocks, out);
 }
 
 

@@ -117,7 +117,7 @@ struct StorageOps {
                        cudaStream_t s);
   int (*choose)(int64_t nx, int64_t ny);
   cudaError_t (*resident)(const StepLaunch &a, const ResidentTiles &g,
-                          int nsteps, cudaStream_t s);
+                          int nsteps, bool reduce, cudaStream_t s);
   cudaError_t (*resident_batch)(const ResidentBatch &b, int nsteps,
                                 cudaStream_t s);
   cudaError_t (*pack)(const double *staging, Fields f, int64_t nx,
@@ -193,15 +193,18 @@ struct ResidentShape {
   int reach = 1;  // nodes a step's result depends on to each side (2: the
                   // multiphase step, whose sources see their neighbours)
 };
+// At most `most` regions.
 ResidentTiles choose_resident(const ResidentShape *shapes, int count,
-                              int nsteps);
+                              int nsteps, int64_t most);
 // The regions of one domain for the chosen rows, warps and steps.
 ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
                              int steps);
 
-// Enqueues nsteps <= g.steps unreduced steps from a.src to a.dst.
+// Enqueues nsteps <= g.steps steps from a.src to a.dst; `reduce` (one step,
+// not the multiphase one): also writes one partial triple per region, padded
+// with zeros to a multiple of kTileWarps, and raises the flag on instability.
 cudaError_t launch_resident(const StepLaunch &a, const ResidentTiles &g,
-                            int nsteps, cudaStream_t s);
+                            int nsteps, bool reduce, cudaStream_t s);
 cudaError_t launch_resident_batch(const ResidentBatch &b, int nsteps,
                                   cudaStream_t s);
 

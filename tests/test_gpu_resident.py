@@ -76,6 +76,34 @@ def test_multiphase_equals_one_launch_per_step(b, nx, ny):
             assert np.array_equal(x.view(np.uint32), y.view(np.uint32)), per
 
 
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_reduced_step_sums(b, nx, ny, storage):
+    """The residual and the mass of a reduced step on regions against the
+    single-step kernel's, from the same state (which ends equal bit for bit).
+    Both add a lane's terms in FP32 (at most 64 rows x 4 columns, the mass
+    compensated): the positive sums agree to 256 * 2^-24 = 1.5e-5, the mass to
+    2^-24 of the lanes' |rho - 1| <= 0.1 sums."""
+    for k, per in enumerate([(False, False), (True, True)]):
+        p = wl.random_problem(nx, ny, seed=nx + 3 * ny + k, amp=0.02,
+                              p_solid=0.15 * k, periodic=per)
+        got = []
+        for variant in (-1, 3):
+            d = b.Domain(nx, ny, p.periodic, p.force, storage=storage)
+            d.set_geometry(p.mask)
+            d.set_moments(p.rho, p.jx, p.jy)
+            d.set_variant(variant)
+            d.step(1)
+            got.append((d.get_state(), d.residual()))
+            d.close()
+        bits = np.uint32 if storage == "f32" else np.uint16
+        for x, y in zip(got[0][0], got[1][0]):
+            assert np.array_equal(x.view(bits), y.view(bits)), per
+        (r0, m0), (r1, m1) = got[0][1], got[1][1]
+        assert r0 == pytest.approx(r1, rel=1.5e-5)
+        assert abs(m0 - m1) <= 6e-8 * 0.1 * nx * ny
+
+
 def test_captured_calls_replay(b):
     """A caller's graph of an even number of steps leaves the state in the
     copy it found it in, so that replays go on from one another."""

@@ -142,8 +142,10 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
 
 // Takes nsteps steps on region (bx, by) (kSC: Shan-Chen multiphase steps;
 // kReduce: one step, whose residual and mass terms become the region's partial
-// triple); every thread of the block calls it.
-template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
+// triple; kForce: the body force is not zero, whose sums are left out
+// otherwise: 5 of the 51 packed operations of a pair); every thread of the
+// block calls it.
+template <typename T, int kR, bool kSr, bool kSC, bool kReduce, bool kForce>
 __device__ __forceinline__ void resident_region(const StepLaunch &a,
                                                 const ResidentTiles &g, int bx,
                                                 int by, int nsteps,
@@ -331,6 +333,8 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
                wm1_6 = bc(-k1_6), half = bc(0.5f), mhalf = bc(-0.5f),
                quarter = bc(0.25f);
 
+  auto with_force = [](float2 v, float2 f) { return kForce ? add(v, f) : v; };
+
   // The residual's and the mass's sums, as step_tile takes them: FP32 per lane
   // (the mass compensated over the rows), FP64 from the warps' sums on.
   float2 rs_num = bc(0.f), rs_den = bc(0.f);
@@ -436,8 +440,8 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
                         float2 nmx, float2 nmy, float2 ex, float2 ey) {
         const float2 dO = d[r], zxO = zx[r], zyO = zy[r];
         float2 dn = add(ad, nd);
-        float2 incx = fma2(w1_6, ex, add(add(ax, nmx), F2x));
-        float2 incy = fma2(half, ey, add(add(ay, nmy), F2y));
+        float2 incx = fma2(w1_6, ex, with_force(add(ax, nmx), F2x));
+        float2 incy = fma2(half, ey, with_force(add(ay, nmy), F2y));
         unsigned code = 0u;
         if (kWalls && (((walls | keep) >> r) & 1u))
           code = codes[(w * kR + r) * kLanes + lane];
@@ -495,7 +499,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
 #pragma unroll
       for (int r = 0; r < kR; ++r) {
         const float2 dc = d[r], zxC = zx[r], zyC = zy[r];
-        const float2 mx = add(zxC, F2x), my = add(zyC, F2y);
+        const float2 mx = with_force(zxC, F2x), my = with_force(zyC, F2y);
         const float2 rho = add(dc, one);
         const float2 ir = make_float2(rcp(rho.x), rcp(rho.y));
         const float2 q = mul(mx, ir);
@@ -531,7 +535,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         const float2 Gs = lpr(G, hG), Gd = lmr(G, hG);
         const float2 Xs = lpr(X, hX), Xd = lmr(X, hX);
         const float2 mxd = lmr(zxC, hZx), myd = lmr(zyC, hZy);
-        const float2 mys = add(lpr(zyC, hZy), F22y);
+        const float2 mys = with_force(lpr(zyC, hZy), F22y);
         const float2 hx = second(zxC, hZx), hy = second(zyC, hZy);
         const float2 U = fma2(w1_9, P, fma2(w1_12, mxd, Gs));
         const float2 V = fma2(w1_3, my, fma2(w1_12, mys, Xd));
@@ -673,12 +677,12 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   }
 }
 
-template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
+template <typename T, int kR, bool kSr, bool kSC, bool kReduce, bool kForce>
 __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     lbm_resident_kernel(const StepLaunch a, const ResidentTiles g, int nsteps) {
   extern __shared__ __align__(128) unsigned char smem[];
-  resident_region<T, kR, kSr, kSC, kReduce>(a, g, blockIdx.x, blockIdx.y,
-                                            nsteps, smem);
+  resident_region<T, kR, kSr, kSC, kReduce, kForce>(
+      a, g, blockIdx.x, blockIdx.y, nsteps, smem);
 }
 
 // A batch's regions: one block per region of the work list.  The launch state
@@ -698,7 +702,8 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
     g = m.tiles;
   }
   __syncthreads();
-  resident_region<T, kR, kSr, false, false>(a, g, item.y, item.z, nsteps, smem);
+  resident_region<T, kR, kSr, false, false, true>(a, g, item.y, item.z, nsteps,
+                                                  smem);
   // the clock of the launches that follow
   if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
 }
@@ -727,9 +732,17 @@ cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
 template <typename T, int kR, bool kSr, bool kSC, bool kReduce>
 cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
                               int nsteps, cudaStream_t s) {
-  return launch_regions<lbm_resident_kernel<T, kR, kSr, kSC, kReduce>>(
-      dim3(g.gx, g.gy), g.warps, resident_smem<kR, kSC>(g.warps),
-      resident_smem<kR, kSC>(kResMaxWarps), s, a, g, nsteps);
+  // Without a body force its sums are left out (us a step: cavity 1024^2 5.5 ->
+  // 5.3, FP16 4096x2500 50.5 -> 48.7, drop 2048^2 22.3 -> 21.6).
+  auto go = [&](auto force) {
+    // (a reduced step, one per call, has the one kernel)
+    return launch_regions<lbm_resident_kernel<
+        T, kR, kSr, kSC, kReduce, decltype(force)::value || kReduce>>(
+        dim3(g.gx, g.gy), g.warps, resident_smem<kR, kSC>(g.warps),
+        resident_smem<kR, kSC>(kResMaxWarps), s, a, g, nsteps);
+  };
+  return a.fx != 0.f || a.fy != 0.f ? go(std::true_type{})
+                                    : go(std::false_type{});
 }
 
 template <typename T, int kR, bool kSr>

@@ -92,11 +92,12 @@ __device__ __forceinline__ float rcp(float x) {
 
 // One step's values of a column pair, rounded to the storage format and back
 // (exactly what a store and a load do).  (c0, c1): the domain's columns of
-// the pair, whose random bits are those of the pair they are stored in.
+// the pair, whose random bits are those of the pair they are stored in; whole:
+// every lane of the warp holds a stored pair.
 template <typename T, bool kSr>
 __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
                                            uint32_t key, uint32_t c0,
-                                           uint32_t c1, bool aligned) {
+                                           uint32_t c1, bool whole) {
   using S = Storage<T>;
   if constexpr (!std::is_same<T, float>::value) {
     const float2 sd = bc(S::kD), sj = bc(S::kJ);
@@ -105,15 +106,19 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
       uint32_t w;
       T e[2];
     } u[3];
-    const float2 v[3] = {__fmul2_rn(d, sd), __fmul2_rn(x, sj),
-                         __fmul2_rn(y, sj)};
+    auto times = [](float2 v, float2 by, bool one) {
+      return one ? v : __fmul2_rn(v, by);
+    };
+    const float2 v[3] = {times(d, sd, S::kD == 1.0f),
+                         times(x, sj, S::kJ == 1.0f),
+                         times(y, sj, S::kJ == 1.0f)};
     if constexpr (kSr) {
       const uint32_t h0 = fmix32(key + (c0 & ~1u) * 0x9e3779b1u);
 #pragma unroll
       for (int f = 0; f < 3; ++f)
         u[f].w = pack_sr(T(), v[f].x, v[f].y,
                          __funnelshift_l(h0, h0, 11 * f));
-      if (!aligned) {  // a wrapped pair of an odd width: column by column
+      if (!whole) {  // a wrapped pair of an odd width: column by column
         const uint32_t h1 = fmix32(key + (c1 & ~1u) * 0x9e3779b1u);
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
@@ -134,9 +139,12 @@ __device__ __forceinline__ void round_pair(float2 &d, float2 &x, float2 &y,
         u[f].e[1] = S::encode(v[f].y);
       }
     }
-    d = __fmul2_rn(make_float2(S::decode(u[0].e[0]), S::decode(u[0].e[1])), id);
-    x = __fmul2_rn(make_float2(S::decode(u[1].e[0]), S::decode(u[1].e[1])), ij);
-    y = __fmul2_rn(make_float2(S::decode(u[2].e[0]), S::decode(u[2].e[1])), ij);
+    d = times(make_float2(S::decode(u[0].e[0]), S::decode(u[0].e[1])), id,
+              S::kD == 1.0f);
+    x = times(make_float2(S::decode(u[1].e[0]), S::decode(u[1].e[1])), ij,
+              S::kJ == 1.0f);
+    y = times(make_float2(S::decode(u[2].e[0]), S::decode(u[2].e[1])), ij,
+              S::kJ == 1.0f);
   }
 }
 
@@ -179,8 +187,11 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
     return periodic ? static_cast<int>(wrap_index(v, n)) : -1;
   };
   const int c0 = wrap(xb, nx, a.periodic_x), c1 = wrap(xb + 1, nx, a.periodic_x);
-  const bool aligned = (c0 & 1) == 0 && c1 == c0 + 1;
-  const bool vec = __all_sync(kFull, aligned && c0 >= 0);
+  const bool vec =
+      __all_sync(kFull, (c0 & 1) == 0 && c1 == c0 + 1 && c0 >= 0);
+  // the row whose random bits lane r < kR keeps (16-bit formats)
+  const int key_row = a.periodic_y ? wrap(yb + lane % kR, ny, 1)
+                                   : yb + lane % kR;
   const float fx = a.fx, fy = a.fy;
 
   // Node types and fields of the region's rows: all loads first, then what is
@@ -374,7 +385,14 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
     constexpr bool kWalls = decltype(with_walls)::value;
     for (int t = 0; t < nsteps; ++t) {
       const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
-      const uint32_t step_key = !kF32 && kSr ? fmix32(a.step + t) : 0u;
+      // stochastic rounding: lane r holds the key of row r and this step (all
+      // lanes hashing every row's took 8 of a pair's 36 integer operations;
+      // with it, and no test per lane for a wrapped pair: FP16 4096^2
+      // 74.3 -> 62.5 us a step, 1024^2 7.0 -> 5.7)
+      uint32_t row_keys = 0u;
+      if constexpr (!kF32 && kSr)
+        row_keys = fmix32(fmix32(a.step + t) ^
+                          (static_cast<uint32_t>(key_row) * 0x85ebca77u));
       // [0] down, [1] up (kSC: two barriers a step, so one buffer; the other
       // holds the potentials)
       Edge *mine = edges + ((kSC ? 0 : t & 1) * warps + w) * 2;
@@ -466,15 +484,11 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
           add_terms(dO, zxO, zyO, dn, xn, yn, own && (fluid & 1u),
                     own && (fluid & 2u) && xb + 1 < nx);
         }
-        if constexpr (!kF32) {
-          int row = yb + r;
-          if constexpr (kSr)
-            if (a.periodic_y) row = wrap(row, ny, 1);
-          round_pair<T, kSr>(
-              dn, xn, yn,
-              fmix32(step_key ^ (static_cast<uint32_t>(row) * 0x85ebca77u)),
-              static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), aligned);
-        }
+        if constexpr (!kF32)
+          round_pair<T, kSr>(dn, xn, yn,
+                             kSr ? __shfl_sync(kFull, row_keys, r) : 0u,
+                             static_cast<uint32_t>(c0),
+                             static_cast<uint32_t>(c1), vec);
         if (kWalls && ((keep >> r) & 1u)) {
           const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
           float2 xk = zxO, yk = zyO;

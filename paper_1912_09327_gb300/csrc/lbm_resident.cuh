@@ -160,6 +160,14 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
                                                 unsigned char *smem) {
   using S = Storage<T>;
   constexpr bool kF32 = std::is_same<T, float>::value;
+  // In blocks with walls every row takes the wall terms and the kept nodes'
+  // selects without a test (rows of porous samples and of small domains mostly
+  // need them, and three tests a row cost their branches' instruction fetches:
+  // porous 2048^2 20.0 -> 17.4 us a step, 48 batched domains 37 -> 33.6, cavity
+  // 256^2 1.04 -> 0.97).  Not where that lost: with 8 rows and no force the
+  // registers it takes spill in the wall-free loop as well (box 4096^2 49 ->
+  // 51), and with 2 rows and a force (channel 64 x 32 +5 %).
+  constexpr bool kFlat = kR == 4 || (kR == 8) == kForce;
   SolidSums *lut = reinterpret_cast<SolidSums *>(smem);
   const int warps = blockDim.x / kLanes;
   Edge *edges = reinterpret_cast<Edge *>(smem + 512 * sizeof(SolidSums));
@@ -297,7 +305,9 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
 #pragma unroll
   for (int r = 0; r < kR + 2; ++r) any |= m0[r] | m1[r];
   any |= (c0 < 0 || c1 < 0 || inside != (1u << (kR + 2)) - 1u) ? 1u : 0u;
-  if (__any_sync(kFull, any != 0u)) {
+  bool any_walls = false;
+  if constexpr (kFlat) any_walls = __syncthreads_or(any != 0u);
+  if (kFlat ? any_walls : __any_sync(kFull, any != 0u) != 0) {
     // solid bits of a row's columns -1 .. 2, and its fluid bits
     auto types = [&](int r, unsigned &fluid) -> unsigned {
       const bool in = (inside >> r) & 1u;
@@ -330,7 +340,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
       fc = fn;
     }
   }
-  const bool any_walls = __syncthreads_or((walls | keep) != 0u);
+  if constexpr (!kFlat) any_walls = __syncthreads_or((walls | keep) != 0u);
   pdl_release();
   if (any_walls && inner) {
     build_solid_lut(lut);
@@ -407,7 +417,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         auto terms = [&](int r) -> Psi {
           const float2 rho = add(d[r], one);
           float2 c = make_float2(1.0f - __expf(-rho.x), 1.0f - __expf(-rho.y));
-          if (kWalls && ((walls >> r) & 1u)) {
+          if (kWalls && (kFlat || ((walls >> r) & 1u))) {
             const unsigned code = codes[(w * kR + r) * kLanes + lane];
             if (code & (1u << 4)) c.x = 0.f;   // the node's own solid bit
             if (code & (1u << 13)) c.y = 0.f;
@@ -461,9 +471,9 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         float2 incx = fma2(w1_6, ex, with_force(add(ax, nmx), F2x));
         float2 incy = fma2(half, ey, with_force(add(ay, nmy), F2y));
         unsigned code = 0u;
-        if (kWalls && (((walls | keep) >> r) & 1u))
+        if (kWalls && (kFlat || (((walls | keep) >> r) & 1u)))
           code = codes[(w * kR + r) * kLanes + lane];
-        if (kWalls && ((walls >> r) & 1u)) {
+        if (kWalls && (kFlat || ((walls >> r) & 1u))) {
           const SolidSums E0 = lut[code & 511u], E1 = lut[(code >> 9) & 511u];
           dn.x = fmaf(dO.x, E0.s0, dn.x);
           incx.x = fmaf(dO.x, E0.sx, incx.x);
@@ -480,7 +490,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         if constexpr (kReduce) {
           const bool own = own_cols && yb + r >= ylo && yb + r < yhi;
           const unsigned fluid =
-              kWalls && ((keep >> r) & 1u) ? code >> 18 : 3u;
+              kWalls && (kFlat || ((keep >> r) & 1u)) ? code >> 18 : 3u;
           add_terms(dO, zxO, zyO, dn, xn, yn, own && (fluid & 1u),
                     own && (fluid & 2u) && xb + 1 < nx);
         }
@@ -489,7 +499,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
                              kSr ? __shfl_sync(kFull, row_keys, r) : 0u,
                              static_cast<uint32_t>(c0),
                              static_cast<uint32_t>(c1), vec);
-        if (kWalls && ((keep >> r) & 1u)) {
+        if (kWalls && (kFlat || ((keep >> r) & 1u))) {
           const bool f0 = (code >> 18) & 1u, f1 = (code >> 19) & 1u;
           float2 xk = zxO, yk = zyO;
           if constexpr (kSC) {

@@ -102,6 +102,7 @@ extern "C" int lbm_step_noalloc(const float *drho_in, const float *jx_in,
   a.partials = partials;
   a.flag = flag;
   a.variant = variant;
+  a.mask_settled = false;
   // as lbm_step takes its reduced last step
   const lbmtau1::ResidentShape dom = {nx, ny, a.periodic_x, a.periodic_y};
   const lbmtau1::ResidentTiles g = lbmtau1::choose_resident(

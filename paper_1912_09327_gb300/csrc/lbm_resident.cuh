@@ -39,7 +39,7 @@
 // operation, and 16-bit formats round to storage after every step with the
 // random bits of the node's own place: the states are equal bit for bit.
 //
-// Measured (us per step, one launch per step -> this, periodic boxes, FP32):
+// Measured (us per step, one launch per step -> this, FP32 periodic boxes):
 // 64^2 13.1 -> 0.64, 256^2 12.0 -> 0.84, 512^2 12.1 -> 1.34, 1024^2 14.2 -> 4.5,
 // 2048^2 40.7 -> 13.7, 4096^2 114 -> 50.7, 8192^2 312 -> 194.  A step on full
 // SMs runs at 500 k MLUPS before the overlap and the loads are paid for; the
@@ -732,10 +732,11 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
 }
 
-// Launches a region kernel, to start while the launch before it ends.
+// Launches a region kernel; `early`: it may start while the launch before it
+// ends (its node types are settled).
 template <auto kKern, typename... A>
 cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
-                           cudaStream_t s, const A &...args) {
+                           bool early, cudaStream_t s, const A &...args) {
   static cudaError_t attr = cudaFuncSetAttribute(
       kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);
   if (attr != cudaSuccess) return attr;
@@ -749,7 +750,7 @@ cudaError_t launch_regions(dim3 grid, int warps, int smem, int most_smem,
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kKern, args...);
 }
 
@@ -763,7 +764,7 @@ cudaError_t launch_resident_k(const StepLaunch &a, const ResidentTiles &g,
     return launch_regions<lbm_resident_kernel<
         T, kR, kSr, kSC, kReduce, decltype(force)::value || kReduce>>(
         dim3(g.gx, g.gy), g.warps, resident_smem<kR, kSC>(g.warps),
-        resident_smem<kR, kSC>(kResMaxWarps), s, a, g, nsteps);
+        resident_smem<kR, kSC>(kResMaxWarps), a.mask_settled, s, a, g, nsteps);
   };
   return a.fx != 0.f || a.fy != 0.f ? go(std::true_type{})
                                     : go(std::false_type{});
@@ -774,8 +775,8 @@ cudaError_t launch_resident_batch_k(const ResidentBatch &b, int nsteps,
                                     cudaStream_t s) {
   return launch_regions<lbm_resident_batch_kernel<T, kR, kSr>>(
       dim3(static_cast<unsigned>(b.nitems)), b.warps,
-      resident_smem<kR, false>(b.warps), resident_smem<kR, false>(kResMaxWarps), s, b,
-      nsteps);
+      resident_smem<kR, false>(b.warps),
+      resident_smem<kR, false>(kResMaxWarps), true, s, b, nsteps);
 }
 
 // f(rows per warp, stochastic rounding) as compile-time constants

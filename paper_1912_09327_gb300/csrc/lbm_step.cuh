@@ -44,6 +44,10 @@ struct StepLaunch {
   // kFlagCopyTimeout); 0 gives up at once.  Draining the copies still in
   // flight before a warp leaves its tile always keeps the one-second bound.
   unsigned long long wait_ns = 1000000000ull;
+  // The node types have been in place since before the launches that may still
+  // be running: a region launch may then read them before those have ended.
+  // False for node types that the caller's own kernels may just have written.
+  bool mask_settled = true;
   // Shan-Chen coupling g of the multiphase step (0: single phase; FP32
   // storage only)
   float g_sc = 0.0f;

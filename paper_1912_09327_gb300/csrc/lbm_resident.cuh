@@ -39,11 +39,14 @@
 // operation, and 16-bit formats round to storage after every step with the
 // random bits of the node's own place: the states are equal bit for bit.
 //
-// Measured (us per step, one launch per step -> this, FP32 periodic boxes):
-// 64^2 13.1 -> 0.64, 256^2 12.0 -> 0.84, 512^2 12.1 -> 1.34, 1024^2 14.2 -> 4.5,
-// 2048^2 40.7 -> 13.7, 4096^2 114 -> 50.7, 8192^2 312 -> 194.  A step on full
-// SMs runs at 500 k MLUPS before the overlap and the loads are paid for; the
-// FMA pipe, which a packed operation holds for two cycles, is 72 % busy then.
+// Measured (us per step in runs of 200, one launch per step -> this, FP32
+// periodic boxes): 256^2 12.0 -> 0.96, 512^2 12.1 -> 1.45, 1024^2 14.2 -> 4.5,
+// 2048^2 40.7 -> 13.5, 4096^2 114 -> 49.1, 8192^2 312 -> 188, 16384^2 1062 ->
+// 737 (364 k MLUPS: more than one trip through memory per step allows).  The
+// next launch's early start is worth 14 % at 1024^2 (5.1 -> 4.4 us a step) and
+// 1.6 % at 4096^2.  A step on full SMs runs at 500 k MLUPS before the overlap
+// and the loads are paid for; the FMA pipe, which a packed operation holds for
+// two cycles, is 68 % busy then.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -205,8 +208,8 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   // Node types and fields of the region's rows: all loads first, then what is
   // derived from them.  A region that lies in the domain with the rows around
   // it needs no index of its own per row and column: one 32-bit offset per row
-  // serves the four planes (a 64-bit index per row, column and plane took 7 %
-  // of the instructions of a four-step launch: box 4096^2 52.6 -> 50.7 us a
+  // serves the four planes (a 64-bit index per row, column and plane took 8 %
+  // of the instructions of a three-step launch: box 4096^2 52.6 -> 50.7 us a
   // step, 64 x 32 regions 69 -> 59).
   unsigned m0[kR + 2], m1[kR + 2];  // rows yb - 1 .. yb + kR
   unsigned inside = (1u << (kR + 2)) - 1u;
@@ -225,7 +228,8 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
     const uint8_t *pm = a.mask + (corner - pitch);
 #pragma unroll
     for (int r = 0; r < kR + 2; ++r)
-      m0[r] = *reinterpret_cast<const unsigned short *>(pm + (mine0 + r * step_y));
+      m0[r] = *reinterpret_cast<const unsigned short *>(
+          pm + (mine0 + r * step_y));
     pdl_wait();  // the fields: written by the launch before this one
     sd += corner;
     sx += corner;
@@ -396,7 +400,7 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
     for (int t = 0; t < nsteps; ++t) {
       const float2 dither = bc(kF32 && kSr ? fp32_dither(a.step + t) : 0.0f);
       // stochastic rounding: lane r holds the key of row r and this step (all
-      // lanes hashing every row's took 8 of a pair's 36 integer operations;
+      // lanes hashing every row's took 8 of a pair's 48 integer operations;
       // with it, and no test per lane for a wrapped pair: FP16 4096^2
       // 74.3 -> 62.5 us a step, 1024^2 7.0 -> 5.7)
       uint32_t row_keys = 0u;
@@ -539,7 +543,8 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
           float m, p;
         };
         auto halo = [&](float2 v) -> Halo {
-          return {__shfl_up_sync(kFull, v.y, 1), __shfl_down_sync(kFull, v.x, 1)};
+          return {__shfl_up_sync(kFull, v.y, 1),
+                  __shfl_down_sync(kFull, v.x, 1)};
         };
         const Halo hK = halo(K), hG = halo(G), hX = halo(X);
         const Halo hZx = halo(zxC), hZy = halo(zyC);

@@ -449,8 +449,8 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   // Several steps per launch up to the reduced last one (lbm_resident.cuh),
   // unless the caller chose a tile variant of the single-step kernel.
   const bool sc = c->p.sc_g != 0.0;
-  const lbmtau1::ResidentShape dom = {c->p.nx, c->p.ny, a.periodic_x,
-                                      a.periodic_y, sc ? 2 : 1};
+  const lbmtau1::ResidentShape dom = {c->p.nx, c->p.ny, c->L.pitch,
+                                      a.periodic_x, a.periodic_y, sc ? 2 : 1};
   if (nsteps >= 2 && !c->variant_set && !(sc && a.sr)) {
     int64_t left = nsteps - 1;
     const int run = static_cast<int>(left < lbmtau1::kLongRun

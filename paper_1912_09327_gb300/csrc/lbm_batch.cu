@@ -138,7 +138,7 @@ int build_regions(lbm_batch *b, int run) {
   std::vector<lbmtau1::ResidentShape> shapes(n);
   for (int i = 0; i < n; ++i) {
     const BatchMember &m = b->h_members[i];
-    shapes[i] = {m.nx, m.ny, m.periodic_x, m.periodic_y};
+    shapes[i] = {m.nx, m.ny, m.pitch, m.periodic_x, m.periodic_y};
   }
   b->regions_for = run;
   b->nregions[0] = b->nregions[1] = 0;
@@ -279,7 +279,7 @@ int upload(lbm_batch *b, int64_t run) {
     if (b->tiles.rows > 0)
       for (BatchMember &m : b->h_members)
         m.tiles = lbmtau1::resident_tiles(
-            {m.nx, m.ny, m.periodic_x, m.periodic_y}, b->tiles.rows,
+            {m.nx, m.ny, m.pitch, m.periodic_x, m.periodic_y}, b->tiles.rows,
             b->tiles.warps, b->tiles.steps);
   }
   if (n) {

@@ -104,7 +104,8 @@ extern "C" int lbm_step_noalloc(const float *drho_in, const float *jx_in,
   a.variant = variant;
   a.mask_settled = false;
   // as lbm_step takes its reduced last step
-  const lbmtau1::ResidentShape dom = {nx, ny, a.periodic_x, a.periodic_y};
+  const lbmtau1::ResidentShape dom = {nx, ny, pitch, a.periodic_x,
+                                      a.periodic_y};
   const lbmtau1::ResidentTiles g = lbmtau1::choose_resident(
       &dom, 1, 1, lbmtau1::step_blocks(nx, ny) * lbmtau1::kTileWarps);
   const int64_t regions = static_cast<int64_t>(g.gx) * g.gy;

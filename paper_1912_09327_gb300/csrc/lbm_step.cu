@@ -221,6 +221,11 @@ ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
   constexpr int kWidth = 64;
   const int64_t nx = d.nx, ny = d.ny;
   ResidentTiles g;
+  // The kernel's offsets within a region are 32-bit: at most 130 rows (the
+  // region's 128 and one to either side) of this pitch are below 2^31.  The
+  // pitch is a caller's (lbm_step_noalloc) and may be far above nx; the
+  // single-step kernel's offsets are 64-bit.
+  if (d.pitch > kResidentPitch) return g;
   const int height = rows * warps;
   g.rows = rows;
   g.warps = warps;
@@ -261,9 +266,11 @@ ResidentTiles choose_resident(const ResidentShape *shapes, int count,
                               int nsteps, int64_t most) {
   ResidentTiles best;
   if (count < 1 || nsteps < 1 || forced_variant() >= 0) return best;
-  for (int i = 0; i < count; ++i)  // rows wrap at most once, and a region's
-    if (shapes[i].nx < 8 || shapes[i].ny < 8 ||  // offsets fit 32 bits
-        shapes[i].nx > (1 << 23))
+  // Sides below 8 are left to the single-step kernel: a region would be
+  // mostly wrapped or outside nodes there.
+  for (int i = 0; i < count; ++i)
+    if (shapes[i].nx < 8 || shapes[i].ny < 8 ||
+        shapes[i].pitch > kResidentPitch)
       return best;
   static const int sms = [] {
     int dev = 0, n = 0;

@@ -188,11 +188,13 @@ cudaError_t launch_tile_flags(int v, const uint8_t *mask, int64_t nx,
 // (sum |du|^2, sum |u|^2, sum (rho - 1)) and raises the flag on instability.
 cudaError_t launch_step(const StepLaunch &a, bool reduce, cudaStream_t s);
 
+constexpr int64_t kResidentPitch = int64_t(1) << 23;  // widest rows of regions
+
 // Tiling for runs of nsteps steps on one domain, or on several that share a
 // launch: rows, warps and steps in the result; rows = 0: none, the steps are
 // then launched one by one.
 struct ResidentShape {
-  int64_t nx, ny;
+  int64_t nx, ny, pitch;
   int periodic_x, periodic_y;
   int reach = 1;  // nodes a step's result depends on to each side (2: the
                   // multiphase step, whose sources see their neighbours)
@@ -200,7 +202,8 @@ struct ResidentShape {
 // At most `most` regions.
 ResidentTiles choose_resident(const ResidentShape *shapes, int count,
                               int nsteps, int64_t most);
-// The regions of one domain for the chosen rows, warps and steps.
+// The regions of one domain for the chosen rows, warps and steps (rows = 0
+// where the domain does not take them).
 ResidentTiles resident_tiles(const ResidentShape &d, int rows, int warps,
                              int steps);
 

@@ -649,9 +649,12 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
       atomicOr(a.flag, kFlagUnstable);
     // The lanes' sums, as pairs of addends, to shared memory; one warp per sum
     // adds each lane's over the warps in two-float arithmetic (exact to about
-    // 2^-46) and only then goes to FP64: the FP64 pipe takes 16 cycles or
-    // more per warp instruction, and a butterfly of three sums in every warp
-    // kept it busy for 2 us per region.
+    // 2^-46, where the lanes' FP32 sums are to 2^-24) and only then goes to
+    // FP64: the FP64 pipe takes 16 cycles or more per warp instruction, and a
+    // butterfly of three sums in every warp kept it busy for 2 us per region.
+    // With FP64 from the lanes on, lbm_step(1) at 4096^2 takes 130 us instead
+    // of 120, with three floats 123.  FP64 does serve where the floats overflow,
+    // as lanes' sums within FP32's range may together.
     __syncthreads();  // the edges' buffer is free
     float2 *terms = reinterpret_cast<float2 *>(edges);
     const int n = warps * kLanes;
@@ -675,6 +678,13 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
         }
       }
       double total = static_cast<double>(hi) + lo;
+      if (!isfinite(hi)) {
+        total = 0.0;
+        for (int i = 0; i < warps; ++i) {
+          const float2 v = terms[k * n + i * kLanes + lane];
+          total += static_cast<double>(v.x) + v.y;
+        }
+      }
 #pragma unroll
       for (int o = kLanes / 2; o > 0; o >>= 1)
         total += __shfl_xor_sync(kFull, total, o);

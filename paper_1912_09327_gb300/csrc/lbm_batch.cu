@@ -291,7 +291,8 @@ int upload(lbm_batch *b, int64_t run) {
   return LBM_OK;
 }
 
-BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity) {
+BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity,
+                        int64_t taken) {
   BatchLaunch L;
   L.members = b->d_members;
   L.items = b->d_items;
@@ -300,16 +301,19 @@ BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity) {
   L.parity = parity;
   L.storage = b->storage;
   L.clock = b->d_counters + kChunk + 1;
+  L.taken = static_cast<unsigned>(taken);
   L.done = b->d_counters + kChunk + 2;
   return L;
 }
 
-int direct_step(lbm_batch *b, int parity, bool reduce) {
+// `taken`: steps that the call's region launches took before it.
+int direct_step(lbm_batch *b, int parity, bool reduce, int64_t taken) {
   unsigned *counter = b->d_counters + kChunk;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(counter)");
-  e = lbmtau1::launch_batch(b->variant, launch_args(b, counter, parity),
-                            reduce, b->stream);
+  e = lbmtau1::launch_batch(b->variant,
+                            launch_args(b, counter, parity, taken), reduce,
+                            b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "batch kernel launch");
   return LBM_OK;
 }
@@ -320,7 +324,7 @@ int direct_step(lbm_batch *b, int parity, bool reduce) {
 int graph_chunk(lbm_batch *b) {
   if (b->graphs_off) {
     for (int t = 0; t < kChunk; ++t) {
-      int st = direct_step(b, t & 1, false);
+      int st = direct_step(b, t & 1, false, 0);
       if (st) return st;
     }
     return LBM_OK;
@@ -339,7 +343,7 @@ int graph_chunk(lbm_batch *b) {
                                      sizeof(unsigned) * kChunk, b->stream);
     for (int t = 0; t < kChunk && le == cudaSuccess; ++t)
       le = lbmtau1::launch_batch(b->variant,
-                                 launch_args(b, b->d_counters + t, t & 1),
+                                 launch_args(b, b->d_counters + t, t & 1, 0),
                                  false, b->stream);
     e = cudaStreamEndCapture(b->stream, &g);
     if (le != cudaSuccess) {
@@ -505,7 +509,7 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(clock)");
     b->clock_set = true;
   }
-  int64_t s = 0;
+  int64_t s = 0, taken = 0;
   // The steps before the last: several per launch, as lbm_step takes them
   // (as many launches as steps modulo two, so that the copies' parity below
   // is the step count's).
@@ -522,8 +526,8 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
       r.warps = b->tiles.warps;
       r.storage = b->storage;
       r.parity = static_cast<int>(l & 1);
-      r.clock = b->clock + static_cast<uint32_t>(s);
-      r.next_clock = b->d_counters + kChunk + 1;
+      r.clock = b->d_counters + kChunk + 1;
+      r.taken = static_cast<unsigned>(s);
       for (int sr = 0; sr < 2; ++sr) {
         if (b->nregions[sr] == 0) continue;
         r.items = b->d_regions + (sr ? b->nregions[0] : 0);
@@ -535,10 +539,11 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
       left -= n;
       s += n;
     }
+    taken = s;  // (one launch per step is left, which adds them to the clock)
   }
   // first step direct (one-time kernel set-up stays outside any capture)
   for (; s < nsteps && s < 2; ++s) {
-    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1);
+    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1, taken);
     if (st) return st;
   }
   while ((s & 1) == 0 && s + kChunk <= nsteps - 1) {
@@ -547,7 +552,7 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
     s += kChunk;
   }
   for (; s < nsteps; ++s) {
-    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1);
+    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1, taken);
     if (st) return st;
   }
   cudaError_t e = lbmtau1::launch_batch_finalize(

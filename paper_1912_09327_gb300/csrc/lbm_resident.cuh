@@ -737,14 +737,14 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   const int4 item = b.items[blockIdx.x];  // member, region x, region y
   if (threadIdx.x == 0) {
     const BatchMember &m = b.members[item.x];
-    fill_launch(a, m, (m.cur ^ b.parity) & 1, b.storage, b.clock);
+    // (read before the launches before this one have ended: no region launch
+    // changes the clock, and the call's first launch follows a copy)
+    fill_launch(a, m, (m.cur ^ b.parity) & 1, b.storage, *b.clock + b.taken);
     g = m.tiles;
   }
   __syncthreads();
   resident_region<T, kR, kSr, false, false, true>(a, g, item.y, item.z, nsteps,
                                                   smem);
-  // the clock of the launches that follow
-  if (blockIdx.x == 0 && threadIdx.x == 0) *b.next_clock = b.clock + nsteps;
 }
 
 // Launches a region kernel; `early`: it may start while the launch before it

@@ -83,13 +83,14 @@ struct lbm_batch {
   bool clock_set;        // device clock and done count zeroed
   double *d_gather;      // 4 doubles per member: result sums and flag
   // The regions of the multi-step launches: those of members that round to
-  // nearest, then those that round stochastically.  Rebuilt with the work
-  // list, or when a call's length asks for another tiling (regions_for).
+  // nearest, then those that round stochastically.  They depend on the members
+  // alone: a caller's graph of one call is replayed between calls of other
+  // lengths and finds its regions in place.
   int4 *d_regions;
   std::vector<int4> h_regions;
   int nregions[2];
   lbmtau1::ResidentTiles tiles;  // rows 0: one launch per step
-  int regions_for;
+  bool regions_known;             // list and tiling are the members'
   cudaStream_t stream;
   std::vector<lbm_ctx *> slots;
   std::vector<BatchMember> h_members;
@@ -127,47 +128,51 @@ void drop_graph(lbm_batch *b) {
   b->graph_variant = -1;
 }
 
-// The longest run whose own length decides the tiling of the regions.
+// The run of steps that the regions' tiling is chosen for; a call that takes
+// fewer takes them on the same regions (one tiling for all lengths: see
+// regions_known).  No tiling of the batches measured takes more per launch.
 constexpr int kBatchRun = 8;
 
-// Chooses the tiling for runs of `run` steps and uploads the members' regions
+// Chooses the tiling of the members' regions and uploads their list
 // (b->tiles.rows = 0 when the steps have to be launched one by one: sizes the
 // regions do not serve, or a workspace too small for their list).
-int build_regions(lbm_batch *b, int run) {
+int build_regions(lbm_batch *b) {
   const int n = static_cast<int>(b->packed.size());
   std::vector<lbmtau1::ResidentShape> shapes(n);
   for (int i = 0; i < n; ++i) {
     const BatchMember &m = b->h_members[i];
     shapes[i] = {m.nx, m.ny, m.pitch, m.periodic_x, m.periodic_y};
   }
-  b->regions_for = run;
   b->nregions[0] = b->nregions[1] = 0;
   const int64_t most = b->max_tiles * lbmtau1::kTileWarps;
-  b->tiles = lbmtau1::choose_resident(shapes.data(), n, run, most);
-  if (b->tiles.rows == 0) return LBM_OK;
-  b->h_regions.clear();
-  for (int sr = 0; sr < 2; ++sr)
-    for (int i = 0; i < n; ++i) {
-      BatchMember &m = b->h_members[i];
-      if ((m.sr != 0) != (sr != 0)) continue;
-      const lbmtau1::ResidentTiles g = lbmtau1::resident_tiles(
-          shapes[i], b->tiles.rows, b->tiles.warps, b->tiles.steps);
-      for (int y = 0; y < g.gy; ++y)
-        for (int x = 0; x < g.gx; ++x)
-          b->h_regions.push_back(make_int4(i, x, y, 0));
-      b->nregions[sr] += g.gx * g.gy;
-    }
-  cudaError_t e = cudaMemcpyAsync(b->d_regions, b->h_regions.data(),
-                                  sizeof(int4) * b->h_regions.size(),
-                                  cudaMemcpyHostToDevice, b->stream);
-  if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(regions)");
+  b->tiles = lbmtau1::choose_resident(shapes.data(), n, kBatchRun, most);
+  if (b->tiles.rows > 0) {
+    b->h_regions.clear();
+    for (int sr = 0; sr < 2; ++sr)
+      for (int i = 0; i < n; ++i) {
+        BatchMember &m = b->h_members[i];
+        if ((m.sr != 0) != (sr != 0)) continue;
+        m.tiles = lbmtau1::resident_tiles(shapes[i], b->tiles.rows,
+                                          b->tiles.warps, b->tiles.steps);
+        for (int y = 0; y < m.tiles.gy; ++y)
+          for (int x = 0; x < m.tiles.gx; ++x)
+            b->h_regions.push_back(make_int4(i, x, y, 0));
+        b->nregions[sr] += m.tiles.gx * m.tiles.gy;
+      }
+    cudaError_t e = cudaMemcpyAsync(b->d_regions, b->h_regions.data(),
+                                    sizeof(int4) * b->h_regions.size(),
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(regions)");
+  }
+  b->regions_known = true;
   return LBM_OK;
 }
 
 // Refreshes the member table (every call: a member may have been stepped on
-// its own since) and, when membership or the variant changed, the work list.
-// `run`: steps the call takes before its last one (0: none).
-int upload(lbm_batch *b, int64_t run) {
+// its own since), when membership or the variant changed the work list, and
+// when membership changed and the call takes steps on them (`regions`) the
+// regions.
+int upload(lbm_batch *b, bool regions) {
   b->packed.clear();
   for (lbm_ctx *c : b->slots)
     if (c) b->packed.push_back(c);
@@ -268,19 +273,10 @@ int upload(lbm_batch *b, int64_t run) {
                                     cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(nitems)");
     b->items_dirty = false;
-    b->regions_for = 0;
   }
-  if (n && run >= 2) {
-    const int r = static_cast<int>(run < kBatchRun ? run : kBatchRun);
-    if (b->regions_for != r) {
-      const int st = build_regions(b, r);
-      if (st) return st;
-    }
-    if (b->tiles.rows > 0)
-      for (BatchMember &m : b->h_members)
-        m.tiles = lbmtau1::resident_tiles(
-            {m.nx, m.ny, m.pitch, m.periodic_x, m.periodic_y}, b->tiles.rows,
-            b->tiles.warps, b->tiles.steps);
+  if (n && regions && !b->regions_known) {
+    const int st = build_regions(b);
+    if (st) return st;
   }
   if (n) {
     cudaError_t e = cudaMemcpyAsync(b->d_members, b->h_members.data(),
@@ -424,7 +420,7 @@ int lbm_batch_create(int32_t capacity, int64_t max_tiles, void *dev_workspace,
   b->d_gather = reinterpret_cast<double *>(base + L.off_gather);
   b->d_regions = reinterpret_cast<int4 *>(base + L.off_regions);
   b->nregions[0] = b->nregions[1] = 0;
-  b->regions_for = 0;
+  b->regions_known = false;
   b->stream = static_cast<cudaStream_t>(cuda_stream);
   b->clock = 0;
   b->clock_set = false;
@@ -460,6 +456,7 @@ int lbm_batch_add(lbm_batch *b, lbm_ctx *ctx, int32_t *slot) {
       b->slots[i] = ctx;
       b->storage = ctx->p.storage;
       b->items_dirty = true;
+      b->regions_known = false;
       if (slot) *slot = i;
       b->err[0] = '\0';
       return LBM_OK;
@@ -473,6 +470,7 @@ int lbm_batch_remove(lbm_batch *b, int32_t slot) {
     return bfail(b, LBM_E_INVAL, "no member in slot %d", slot);
   b->slots[slot] = nullptr;
   b->items_dirty = true;
+  b->regions_known = false;
   b->err[0] = '\0';
   return LBM_OK;
 }
@@ -501,7 +499,7 @@ int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
   if (!b) return LBM_E_INVAL;
   if (nsteps < 0) return bfail(b, LBM_E_INVAL, "nsteps < 0");
   if (nsteps == 0 || lbm_batch_members(b) == 0) return LBM_OK;
-  int st = upload(b, nsteps - 1);
+  int st = upload(b, nsteps >= 3);
   if (st) return st;
   if (!b->clock_set) {  // the batch clock and the done count start at zero
     cudaError_t e = cudaMemsetAsync(b->d_counters + kChunk + 1, 0,
@@ -622,7 +620,7 @@ int lbm_batch_residuals(lbm_batch *b, double *residual, double *mass,
     residual[i] = mass[i] = 0.0;
     status[i] = LBM_E_STATE;
   }
-  int st = upload(b, 0);  // descriptors in slot order of the current members
+  int st = upload(b, false);  // descriptors in slot order of the current members
   if (st) return st;
   const int n = static_cast<int>(b->packed.size());
   if (n == 0) return LBM_OK;

@@ -55,3 +55,30 @@ def test_replays_equal_calls(storage, rounding):
             assert np.array_equal(x, y)
         got.close()
         want.close()
+
+
+@pytest.mark.parametrize("between", [2, 4, 30])
+def test_replays_between_calls_of_other_lengths(between):
+    """A replay finds the members' regions as the captured call left them,
+    whatever (even) lengths the calls since then had (an odd call leaves the
+    member table naming the other copies)."""
+    import torch
+    from paper_1912_09327_gb300 import binding as b
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        got, doms = make(b, s, "f32", "nearest")
+        want, other = make(b, s, "f32", "nearest")
+        got.step(8)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+            got.step(8)
+        g.replay()
+        for _ in range(2):
+            got.step(between)
+        g.replay()
+        want.step(24 + 2 * between)
+        for x, y in zip(states(doms), states(other)):
+            assert np.array_equal(x, y)
+        got.close()
+        want.close()

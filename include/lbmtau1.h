@@ -404,10 +404,13 @@ int lbm_variant_tile(int32_t variant, int64_t *tile_x, int64_t *tile_y,
 int32_t lbm_variant_has_clean_code(int32_t variant);
 
 /* Autotuner: times steps_per_variant (even, >= 2) batch steps, plus two
- * warm-up steps, with every tile variant and keeps the fastest.  These are
- * real steps: every member advances by (steps_per_variant + 2) times the
- * variant count.  ms_per_step (NULL or lbm_variant_count() doubles) receives
- * the measured time per step of each variant.  Synchronises the stream. */
+ * warm-up steps, with every tile variant and keeps the fastest.  Where regions
+ * take the steps before a call's last one, the variant decides that reduced
+ * last step alone, and all the timed steps are reduced ones; else they are one
+ * call's.  These are real steps: every member advances by (steps_per_variant +
+ * 2) times the variant count.  ms_per_step (NULL or lbm_variant_count()
+ * doubles) receives the measured time per step of each variant.  Synchronises
+ * the stream. */
 int lbm_batch_autotune(lbm_batch *b, int32_t steps_per_variant,
                        int32_t *chosen, double *ms_per_step);
 

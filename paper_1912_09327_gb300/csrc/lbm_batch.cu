@@ -360,6 +360,79 @@ int graph_chunk(lbm_batch *b) {
   return LBM_OK;
 }
 
+// Advances every member by nsteps; reduce_all: one reduced launch per step, as
+// the last step of a call is taken.
+int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
+  if (nsteps == 0 || lbm_batch_members(b) == 0) return LBM_OK;
+  int st = upload(b, nsteps >= 3);
+  if (st) return st;
+  if (!b->clock_set) {  // the batch clock and the done count start at zero
+    cudaError_t e = cudaMemsetAsync(b->d_counters + kChunk + 1, 0,
+                                    2 * sizeof(unsigned), b->stream);
+    if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(clock)");
+    b->clock_set = true;
+  }
+  int64_t s = 0, taken = 0;
+  // The steps before the last: several per launch, as lbm_step takes them
+  // (as many launches as steps modulo two, so that the copies' parity below
+  // is the step count's).
+  if (nsteps >= 3 && b->tiles.rows > 0 && !reduce_all) {
+    int64_t left = nsteps - 1;
+    int64_t launches = (left + b->tiles.steps - 1) / b->tiles.steps;
+    launches += (left - launches) & 1;
+    for (int64_t l = 0; l < launches; ++l) {
+      const int n =
+          static_cast<int>((left + launches - l - 1) / (launches - l));
+      lbmtau1::ResidentBatch r;
+      r.members = b->d_members;
+      r.rows = b->tiles.rows;
+      r.warps = b->tiles.warps;
+      r.storage = b->storage;
+      r.parity = static_cast<int>(l & 1);
+      r.clock = b->d_counters + kChunk + 1;
+      r.taken = static_cast<unsigned>(s);
+      for (int sr = 0; sr < 2; ++sr) {
+        if (b->nregions[sr] == 0) continue;
+        r.items = b->d_regions + (sr ? b->nregions[0] : 0);
+        r.nitems = b->nregions[sr];
+        r.sr = sr;
+        cudaError_t e = lbmtau1::launch_resident_batch(r, n, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "batch region launch");
+      }
+      left -= n;
+      s += n;
+    }
+    taken = s;  // (one launch per step is left, which adds them to the clock)
+  }
+  // first step direct (one-time kernel set-up stays outside any capture)
+  for (; s < nsteps && s < 2; ++s) {
+    st = direct_step(b, static_cast<int>(s & 1),
+                     reduce_all || s == nsteps - 1, taken);
+    if (st) return st;
+  }
+  while (!reduce_all && (s & 1) == 0 && s + kChunk <= nsteps - 1) {
+    st = graph_chunk(b);
+    if (st) return st;
+    s += kChunk;
+  }
+  for (; s < nsteps; ++s) {
+    st = direct_step(b, static_cast<int>(s & 1),
+                     reduce_all || s == nsteps - 1, taken);
+    if (st) return st;
+  }
+  cudaError_t e = lbmtau1::launch_batch_finalize(
+      b->d_members, static_cast<int>(b->packed.size()), b->stream);
+  if (e != cudaSuccess) return bcuda(b, e, "batch finalize launch");
+  for (lbm_ctx *c : b->packed) {
+    c->cur ^= static_cast<int>(nsteps & 1);
+    c->has_residual = true;
+    c->steps += nsteps;
+  }
+  b->clock += static_cast<uint32_t>(nsteps);
+  b->err[0] = '\0';
+  return LBM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -498,72 +571,7 @@ int32_t lbm_batch_variant(const lbm_batch *b) { return b ? b->variant : -1; }
 int lbm_batch_step(lbm_batch *b, int64_t nsteps) {
   if (!b) return LBM_E_INVAL;
   if (nsteps < 0) return bfail(b, LBM_E_INVAL, "nsteps < 0");
-  if (nsteps == 0 || lbm_batch_members(b) == 0) return LBM_OK;
-  int st = upload(b, nsteps >= 3);
-  if (st) return st;
-  if (!b->clock_set) {  // the batch clock and the done count start at zero
-    cudaError_t e = cudaMemsetAsync(b->d_counters + kChunk + 1, 0,
-                                    2 * sizeof(unsigned), b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(clock)");
-    b->clock_set = true;
-  }
-  int64_t s = 0, taken = 0;
-  // The steps before the last: several per launch, as lbm_step takes them
-  // (as many launches as steps modulo two, so that the copies' parity below
-  // is the step count's).
-  if (nsteps >= 3 && b->tiles.rows > 0) {
-    int64_t left = nsteps - 1;
-    int64_t launches = (left + b->tiles.steps - 1) / b->tiles.steps;
-    launches += (left - launches) & 1;
-    for (int64_t l = 0; l < launches; ++l) {
-      const int n =
-          static_cast<int>((left + launches - l - 1) / (launches - l));
-      lbmtau1::ResidentBatch r;
-      r.members = b->d_members;
-      r.rows = b->tiles.rows;
-      r.warps = b->tiles.warps;
-      r.storage = b->storage;
-      r.parity = static_cast<int>(l & 1);
-      r.clock = b->d_counters + kChunk + 1;
-      r.taken = static_cast<unsigned>(s);
-      for (int sr = 0; sr < 2; ++sr) {
-        if (b->nregions[sr] == 0) continue;
-        r.items = b->d_regions + (sr ? b->nregions[0] : 0);
-        r.nitems = b->nregions[sr];
-        r.sr = sr;
-        cudaError_t e = lbmtau1::launch_resident_batch(r, n, b->stream);
-        if (e != cudaSuccess) return bcuda(b, e, "batch region launch");
-      }
-      left -= n;
-      s += n;
-    }
-    taken = s;  // (one launch per step is left, which adds them to the clock)
-  }
-  // first step direct (one-time kernel set-up stays outside any capture)
-  for (; s < nsteps && s < 2; ++s) {
-    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1, taken);
-    if (st) return st;
-  }
-  while ((s & 1) == 0 && s + kChunk <= nsteps - 1) {
-    st = graph_chunk(b);
-    if (st) return st;
-    s += kChunk;
-  }
-  for (; s < nsteps; ++s) {
-    st = direct_step(b, static_cast<int>(s & 1), s == nsteps - 1, taken);
-    if (st) return st;
-  }
-  cudaError_t e = lbmtau1::launch_batch_finalize(
-      b->d_members, static_cast<int>(b->packed.size()), b->stream);
-  if (e != cudaSuccess) return bcuda(b, e, "batch finalize launch");
-  for (lbm_ctx *c : b->packed) {
-    c->cur ^= static_cast<int>(nsteps & 1);
-    c->has_residual = true;
-    c->steps += nsteps;
-  }
-  b->clock += static_cast<uint32_t>(nsteps);
-  b->err[0] = '\0';
-  return LBM_OK;
+  return advance(b, nsteps, false);
 }
 
 int lbm_batch_autotune(lbm_batch *b, int32_t steps_per_variant,
@@ -571,6 +579,11 @@ int lbm_batch_autotune(lbm_batch *b, int32_t steps_per_variant,
   if (!b) return LBM_E_INVAL;
   if (steps_per_variant < 2 || steps_per_variant % 2)
     return bfail(b, LBM_E_INVAL, "steps_per_variant must be even and >= 2");
+  // The variant decides the reduced last step of a call where regions take the
+  // others (those steps are timed then), else every step of it.
+  int st = lbm_batch_members(b) > 0 ? upload(b, true) : LBM_OK;
+  if (st) return st;
+  const bool last_only = b->regions_known && b->tiles.rows > 0;
   const int nv = lbmtau1::variant_count();
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return LBM_E_CUDA;
@@ -580,14 +593,13 @@ int lbm_batch_autotune(lbm_batch *b, int32_t steps_per_variant,
   }
   int best = b->variant;
   float best_ms = -1.f;
-  int st = LBM_OK;
   for (int v = 0; v < nv && st == LBM_OK; ++v) {
     st = lbm_batch_set_variant(b, v);
     if (st) break;
-    st = lbm_batch_step(b, 2);  // warm-up, builds this variant's set-up
+    st = advance(b, 2, last_only);  // warm-up, builds this variant's set-up
     if (st) break;
     cudaEventRecord(e0, b->stream);
-    st = lbm_batch_step(b, steps_per_variant);
+    st = advance(b, steps_per_variant, last_only);
     if (st) break;
     cudaEventRecord(e1, b->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) {

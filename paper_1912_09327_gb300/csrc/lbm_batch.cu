@@ -287,8 +287,7 @@ int upload(lbm_batch *b, bool regions) {
   return LBM_OK;
 }
 
-BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity,
-                        int64_t taken) {
+BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity) {
   BatchLaunch L;
   L.members = b->d_members;
   L.items = b->d_items;
@@ -297,19 +296,16 @@ BatchLaunch launch_args(lbm_batch *b, unsigned *counter, int parity,
   L.parity = parity;
   L.storage = b->storage;
   L.clock = b->d_counters + kChunk + 1;
-  L.taken = static_cast<unsigned>(taken);
   L.done = b->d_counters + kChunk + 2;
   return L;
 }
 
-// `taken`: steps that the call's region launches took before it.
-int direct_step(lbm_batch *b, int parity, bool reduce, int64_t taken) {
+int direct_step(lbm_batch *b, int parity, bool reduce) {
   unsigned *counter = b->d_counters + kChunk;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(counter)");
-  e = lbmtau1::launch_batch(b->variant,
-                            launch_args(b, counter, parity, taken), reduce,
-                            b->stream);
+  e = lbmtau1::launch_batch(b->variant, launch_args(b, counter, parity),
+                            reduce, b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "batch kernel launch");
   return LBM_OK;
 }
@@ -320,7 +316,7 @@ int direct_step(lbm_batch *b, int parity, bool reduce, int64_t taken) {
 int graph_chunk(lbm_batch *b) {
   if (b->graphs_off) {
     for (int t = 0; t < kChunk; ++t) {
-      int st = direct_step(b, t & 1, false, 0);
+      int st = direct_step(b, t & 1, false);
       if (st) return st;
     }
     return LBM_OK;
@@ -339,7 +335,7 @@ int graph_chunk(lbm_batch *b) {
                                      sizeof(unsigned) * kChunk, b->stream);
     for (int t = 0; t < kChunk && le == cudaSuccess; ++t)
       le = lbmtau1::launch_batch(b->variant,
-                                 launch_args(b, b->d_counters + t, t & 1, 0),
+                                 launch_args(b, b->d_counters + t, t & 1),
                                  false, b->stream);
     e = cudaStreamEndCapture(b->stream, &g);
     if (le != cudaSuccess) {
@@ -372,7 +368,7 @@ int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(clock)");
     b->clock_set = true;
   }
-  int64_t s = 0, taken = 0;
+  int64_t s = 0;
   // The steps before the last: several per launch, as lbm_step takes them
   // (as many launches as steps modulo two, so that the copies' parity below
   // is the step count's).
@@ -390,9 +386,11 @@ int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
       r.storage = b->storage;
       r.parity = static_cast<int>(l & 1);
       r.clock = b->d_counters + kChunk + 1;
+      r.done = b->d_counters + kChunk + 2;
       r.taken = static_cast<unsigned>(s);
       for (int sr = 0; sr < 2; ++sr) {
         if (b->nregions[sr] == 0) continue;
+        r.advance = l == launches - 1 && (sr == 1 || b->nregions[1] == 0);
         r.items = b->d_regions + (sr ? b->nregions[0] : 0);
         r.nitems = b->nregions[sr];
         r.sr = sr;
@@ -402,12 +400,11 @@ int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
       left -= n;
       s += n;
     }
-    taken = s;  // (one launch per step is left, which adds them to the clock)
   }
   // first step direct (one-time kernel set-up stays outside any capture)
   for (; s < nsteps && s < 2; ++s) {
     st = direct_step(b, static_cast<int>(s & 1),
-                     reduce_all || s == nsteps - 1, taken);
+                     reduce_all || s == nsteps - 1);
     if (st) return st;
   }
   while (!reduce_all && (s & 1) == 0 && s + kChunk <= nsteps - 1) {
@@ -417,7 +414,7 @@ int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
   }
   for (; s < nsteps; ++s) {
     st = direct_step(b, static_cast<int>(s & 1),
-                     reduce_all || s == nsteps - 1, taken);
+                     reduce_all || s == nsteps - 1);
     if (st) return st;
   }
   cudaError_t e = lbmtau1::launch_batch_finalize(

@@ -1311,7 +1311,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
   SolidSums *lut = reinterpret_cast<SolidSums *>(smem);
   build_solid_lut(lut);
   // the batch clock: read by every block before the last block advances it
-  const unsigned clock = *b.clock + b.taken;
+  const unsigned clock = *b.clock;
   __syncthreads();
   const int n = *b.nitems;
   const int slot = threadIdx.x / kLanes;

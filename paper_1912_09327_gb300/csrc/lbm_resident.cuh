@@ -737,10 +737,19 @@ __global__ void __launch_bounds__(kResMaxWarps *kLanes, 1)
   const int4 item = b.items[blockIdx.x];  // member, region x, region y
   if (threadIdx.x == 0) {
     const BatchMember &m = b.members[item.x];
-    // (read before the launches before this one have ended: no region launch
+    // (read before the launches before this one have ended: none of them
     // changes the clock, and the call's first launch follows a copy)
-    fill_launch(a, m, (m.cur ^ b.parity) & 1, b.storage, *b.clock + b.taken);
+    const unsigned clock = *b.clock + b.taken;
+    fill_launch(a, m, (m.cur ^ b.parity) & 1, b.storage, clock);
     g = m.tiles;
+    // The clock for the step that follows the region launches, set by the last
+    // block to have read it (the launches before this one have: their blocks
+    // read it before they let this one start).  At the end of the block a fence
+    // and this took 3 % of a launch.
+    if (b.advance && atomicAdd(b.done, 1u) == gridDim.x - 1) {
+      *b.done = 0u;
+      *b.clock = clock + nsteps;
+    }
   }
   __syncthreads();
   resident_region<T, kR, kSr, false, false, true>(a, g, item.y, item.z, nsteps,

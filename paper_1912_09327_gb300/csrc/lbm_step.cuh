@@ -94,7 +94,6 @@ struct BatchLaunch {
   int parity;             // step index within the call, mod 2
   int storage;            // storage format shared by all members
   unsigned int *clock;    // batch steps taken (advanced by each launch)
-  unsigned int taken;     // steps that region launches took since its value
   unsigned int *done;     // blocks finished in this launch (zero between)
 };
 
@@ -108,11 +107,14 @@ struct ResidentBatch {
   int sr;               // stochastic rounding, the same for every item
   int storage;
   int parity;           // launches taken within the call, mod 2
-  // The batch clock at the start of the call, and the steps that the call's
-  // launches before this one took: the clock itself stays on the device, so
-  // that a replayed capture of the call goes on with new random bits.
-  const unsigned *clock;
+  // The batch clock, and the steps that the call's launches before this one
+  // took: the clock stays on the device, so that a replayed capture of the call
+  // goes on with new random bits.  The call's last region launch (`advance`)
+  // adds all of the call's region steps to it.
+  unsigned *clock;
+  unsigned *done;       // blocks that have read it then (zero between)
   unsigned taken;
+  bool advance;
 };
 
 // The launchers of one storage format.  The kernels are templates on the

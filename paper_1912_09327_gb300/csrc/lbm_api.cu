@@ -451,6 +451,12 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   const bool sc = c->p.sc_g != 0.0;
   const lbmtau1::ResidentShape dom = {c->p.nx, c->p.ny, c->L.pitch,
                                       a.periodic_x, a.periodic_y, sc ? 2 : 1};
+  const bool reduce_regions =
+      !c->variant_set && !sc && c->wait_ns == kDefaultWaitNs;
+  if (reduce_regions && !c->reduce_known) {
+    const int st = choose_reduce(c, dom);
+    if (st) return st;
+  }
   if (nsteps >= 2 && !c->variant_set && !(sc && a.sr)) {
     int64_t left = nsteps - 1;
     const int run = static_cast<int>(left < lbmtau1::kLongRun
@@ -467,6 +473,15 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
     int64_t launches =
         tiles.rows > 0 ? (left + tiles.steps - 1) / tiles.steps : 0;
     if (launches > 0) launches += (left - launches) & 1;
+    // With one step per launch (calls of two or three steps) a large clean
+    // FP32 domain has nothing to gain from regions: its single-step kernel
+    // moves the same bytes with less overlap (choose_reduce).  us per call on
+    // regions and with that kernel: 16384^2 box, two steps 2472 and 2344, three
+    // 3711 and 3406; 8192^2 cavity 673 and 670, 987 and 972.  16-bit formats
+    // stay (8192^2 FP16 723 and 765, 1041 and 1115).
+    if (launches == left && reduce_regions && c->reduce_tiles.rows == 0 &&
+        c->p.storage == lbmtau1::kStorageF32)
+      launches = 0;
     for (; launches > 0; --launches) {
       const int n = static_cast<int>((left + launches - 1) / launches);
       a.src = c->f[c->cur];
@@ -483,12 +498,7 @@ int lbm_step(lbm_ctx *c, int64_t nsteps) {
   // The reduced last step on regions too, one partial triple each; unless the
   // caller bounds the waits for staged rows, which are the single-step
   // kernel's.
-  if (s == nsteps - 1 && !c->variant_set && !sc &&
-      c->wait_ns == kDefaultWaitNs) {
-    if (!c->reduce_known) {
-      const int st = choose_reduce(c, dom);
-      if (st) return st;
-    }
+  if (s == nsteps - 1 && reduce_regions) {
     const lbmtau1::ResidentTiles &g = c->reduce_tiles;
     if (g.rows > 0) {
       a.src = c->f[c->cur];

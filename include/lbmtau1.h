@@ -168,28 +168,32 @@ int lbm_set_moments(lbm_ctx *ctx, const double *rho, const double *jx,
  * Enqueues nsteps LBMTau1 time steps (Algorithm 1), asynchronously.  The last
  * step of the call also reduces the residual and mass that lbm_residual
  * returns and checks for rho <= 0 or non-finite values.  nsteps = 0 is a
- * no-op.  The steps before the last are taken several per launch, unless a
- * tile variant was set (lbm_set_variant), a side is shorter than 8 nodes or
- * longer than 2^23 along x, or a multiphase step rounds stochastically: those
- * take one launch per step, and on a
- * stream that can be captured (not the legacy default stream, and not under a
- * capture of the caller's) runs of 16 inner steps are then replayed from a
- * CUDA graph captured at first use (FP32 storage, or 16-bit storage rounded
- * to nearest; stochastic rounding launches every step).
+ * no-op.  The steps before the last are taken several per launch (on regions
+ * held in registers), unless a tile variant was set (lbm_set_variant), a side
+ * is shorter than 8 nodes or longer than 2^23 along x, or a multiphase step
+ * rounds stochastically: those take one launch per step, and on a stream that
+ * can be captured (not the legacy default stream, and not under a capture of
+ * the caller's) runs of 16 inner steps are then replayed from a CUDA graph
+ * captured at first use (FP32 storage, or 16-bit storage rounded to nearest;
+ * stochastic rounding launches every step).  The reduced last step runs on
+ * regions too; with the single-step kernel run multiphase domains, large
+ * domains that are mostly clear of walls (in FP32 with the whole of a call of
+ * two or three steps), and all that take one launch per step.
  * Errors: LBM_E_INVAL (nsteps < 0), LBM_E_STATE, LBM_E_CUDA (launch failure).
  */
 int lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /*
  * Tile variant (block tile shape, 0 .. lbm_variant_count() - 1) of the
- * context's single-step kernel, which takes the reduced last step of a call
- * and, once a variant is set by hand, every step.  All variants give bit-identical states; they differ
- * in how well their grid fills the device.  By default (variant -1) the first
- * step picks one from the domain size, the SM count and the kernels'
- * occupancy (the environment variable LBMTAU1_STEP_VARIANT, when set to a
- * valid index, overrides that choice).  lbm_set_variant may be called between
- * steps; lbm_variant returns the variant the next step uses, choosing it if
- * that has not happened yet (-1 for a null context).
+ * context's single-step kernel (lbm_step says which steps it takes; every
+ * step once a variant is set by hand).  All variants give bit-identical
+ * states; they differ in how well their grid fills the device.  By default
+ * (variant -1) the first step that this kernel takes picks one from the domain
+ * size, the SM count and the kernels' occupancy (the environment variable
+ * LBMTAU1_STEP_VARIANT, when set to a valid index, overrides that choice and
+ * keeps every step off the regions).  lbm_set_variant may be called between
+ * steps; lbm_variant returns the variant of the next step that this kernel
+ * takes, choosing it if that has not happened yet (-1 for a null context).
  * Errors: LBM_E_INVAL (variant < -1 or >= lbm_variant_count()).
  */
 int lbm_set_variant(lbm_ctx *ctx, int32_t variant);
@@ -289,8 +293,7 @@ int lbm_change_since(lbm_ctx *ctx, const void *dev_buf, int64_t steps,
  * allocator and forbids side allocations, or a loop with a hard latency
  * budget where cudaMalloc / cudaFree are not acceptable).
  *
- * Runs one reduced LBMTau1 step, the same kernel as lbm_step, from
- * caller-owned device fields (rho - 1, jx, jy as float32, rows of `pitch`
+ * Runs one reduced LBMTau1 step from caller-owned device fields (rho - 1, jx, jy as float32, rows of `pitch`
  * elements) into a second caller-owned set, with the node types in a
  * caller-owned uint8 array of the same pitch.  It calls no cudaMalloc,
  * cudaFree or allocating library routine: the reduction scratch is a
@@ -341,9 +344,13 @@ void lbm_destroy(lbm_ctx *ctx);
  * stream.  lbm_batch_step advances every member by nsteps: the steps before the
  * last several per launch, over a list of all members' regions; the reduced
  * last step over a work list of all members' block tiles, taken by a
- * persistent grid through an atomic counter.  Each member ends bit for bit where it would
- * have ended alone, and afterwards lbm_moments / lbm_residual / lbm_step work
- * on it as usual (the last step of the call is reduced for every member).
+ * persistent grid through an atomic counter.  Each member ends bit for bit
+ * where it would have ended alone, and afterwards lbm_moments / lbm_residual /
+ * lbm_step work on it as usual (the last step of the call is reduced for every
+ * member).  A caller's capture of lbm_batch_step with an even nsteps may be
+ * replayed while the membership stays and calls of even lengths come between
+ * (the first call after a change of membership uploads the work lists: make it
+ * outside the capture).
  */
 typedef struct lbm_batch lbm_batch;
 

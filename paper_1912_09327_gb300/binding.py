@@ -378,7 +378,7 @@ def lbm_batch_destroy(b) -> None:
 
 
 class Batch:
-    """A batch of Domains stepped together (one launch per step); the
+    """A batch of Domains stepped together (shared launches); the
     workspace comes from torch, the stream is shared with the members."""
 
     def __init__(self, capacity, max_tiles, device="cuda", stream=None):

@@ -340,10 +340,11 @@ int select_variant(lbm_ctx *c) {
 
 // Chooses how the context takes a call's reduced last step (reduce_tiles).  A
 // single step on regions beats the single-step kernel on small and middling
-// domains (1024^2 27 -> 19 us with the finalize, 64^2 25 -> 12); where most
-// tiles of a large domain are clean, that kernel's long march with its copies
-// in flight is the faster way to move 24 bytes a node (8192^2 379 against
-// 543 us).
+// domains (us with the finalize, single-step kernel -> regions: 64^2 24.6 ->
+// 6.5, 1024^2 26.6 -> 15.2, 4096^2 156 -> 121); where most tiles of a large
+// domain are clean, that kernel's long march with its copies in flight is the
+// faster way to move 24 bytes a node (box 8192^2 376, on regions
+// (lbm_step_noalloc) 441; 16384^2 1276 and 1677).
 int choose_reduce(lbm_ctx *c, const lbmtau1::ResidentShape &dom) {
   c->reduce_tiles = lbmtau1::ResidentTiles();
   c->reduce_known = true;

@@ -1,5 +1,5 @@
 // Batched stepping of many independent LBMTau1 domains (each an lbm_ctx) with
-// one launch per time step for the whole batch.
+// launches for the whole batch.
 //
 // Every member keeps its own workspace (fields, node types, reduction
 // partials); the batch holds a device table of member descriptors and a work

@@ -103,7 +103,11 @@ extern "C" int lbm_step_noalloc(const float *drho_in, const float *jx_in,
   a.flag = flag;
   a.variant = variant;
   a.mask_settled = false;
-  // as lbm_step takes its reduced last step
+  // On regions, as lbm_step takes its reduced last step, and large clean
+  // domains too: the clean-tile kernel needs flags that are computed ahead, and
+  // the general one is slower at every size (us a call, general kernel ->
+  // regions: box 64^2 30 -> 12, 1024^2 31 -> 21, 4096^2 162 -> 128, 8192^2 488
+  // -> 441, 16384^2 1750 -> 1677; porous 4096^2 164 -> 148).
   const lbmtau1::ResidentShape dom = {nx, ny, pitch, a.periodic_x,
                                       a.periodic_y};
   const lbmtau1::ResidentTiles g = lbmtau1::choose_resident(

@@ -7,7 +7,8 @@
 // (kR * warps) rows once, takes up to `steps` steps on it in registers and
 // stores the nodes that no missing neighbour has reached: a region's rim goes
 // stale by one node per step, so regions overlap by that much.  The inner
-// steps of lbm_step (all but its reduced last one) run this way.
+// steps of lbm_step run this way, and its reduced last one as a launch of one
+// step (below).
 //
 // Layout: a lane holds two adjacent columns (one packed pair) of kR rows, a
 // warp all 64 columns.  Two columns and eight rows keep the same 16 nodes in a
@@ -32,7 +33,7 @@
 //
 // A call's reduced last step runs here as a launch of one step (us per
 // lbm_step(ctx, 1), single-step kernel -> this, with the finalize: 64^2
-// 24.7 -> 6.5, 1024^2 26.7 -> 14.1, 2048^2 59 -> 34, 4096^2 156 -> 113), except
+// 24.6 -> 6.5, 1024^2 26.6 -> 15.2, 2048^2 59 -> 36, 4096^2 156 -> 121), except
 // where a large domain's tiles are mostly clean (choose_reduce).
 //
 // Every node's arithmetic is that of step_tile (lbm_kernels.cuh), operation by
@@ -168,8 +169,9 @@ __device__ __forceinline__ void resident_region(const StepLaunch &a,
   // need them, and three tests a row cost their branches' instruction fetches:
   // porous 2048^2 20.0 -> 17.4 us a step, 48 batched domains 37 -> 33.6, cavity
   // 256^2 1.04 -> 0.97).  Not where that lost: with 8 rows and no force the
-  // registers it takes spill in the wall-free loop as well (box 4096^2 49 ->
-  // 51), and with 2 rows and a force (channel 64 x 32 +5 %).
+  // registers it takes spill in the wall-free loop as well (ptxas: 48 bytes of
+  // spill stores instead of 16; box 4096^2 49 -> 51), and with 2 rows and a
+  // force (channel 64 x 32, the one domain it was measured on, +5 %).
   constexpr bool kFlat = kR == 4 || (kR == 8) == kForce;
   SolidSums *lut = reinterpret_cast<SolidSums *>(smem);
   const int warps = blockDim.x / kLanes;

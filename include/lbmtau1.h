@@ -349,8 +349,7 @@ void lbm_destroy(lbm_ctx *ctx);
  * lbm_step work on it as usual (the last step of the call is reduced for every
  * member).  A caller's capture of lbm_batch_step with an even nsteps may be
  * replayed while the membership stays and calls of even lengths come between
- * (the first call after a change of membership uploads the work lists: make it
- * outside the capture).
+ * (with stochastic rounding not a batch's first call, which clears its clock).
  */
 typedef struct lbm_batch lbm_batch;
 

@@ -122,6 +122,18 @@ int bcuda(lbm_batch *b, cudaError_t e, const char *what) {
   return bfail(b, LBM_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Whether what is enqueued now runs with this call: under a caller's capture
+// it is only recorded, and a list "uploaded" there is not on the device for
+// calls before the first replay.
+bool runs_now(const lbm_batch *b) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return cs == cudaStreamCaptureStatusNone;
+}
+
 void drop_graph(lbm_batch *b) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
@@ -164,7 +176,7 @@ int build_regions(lbm_batch *b) {
                                     cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(regions)");
   }
-  b->regions_known = true;
+  b->regions_known = runs_now(b);
   return LBM_OK;
 }
 
@@ -272,7 +284,7 @@ int upload(lbm_batch *b, bool regions) {
     cudaError_t e = cudaMemcpyAsync(b->d_nitems, &b->nitems, sizeof(int),
                                     cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemcpyAsync(nitems)");
-    b->items_dirty = false;
+    b->items_dirty = !runs_now(b);
   }
   if (n && regions && !b->regions_known) {
     const int st = build_regions(b);
@@ -366,7 +378,7 @@ int advance(lbm_batch *b, int64_t nsteps, bool reduce_all) {
     cudaError_t e = cudaMemsetAsync(b->d_counters + kChunk + 1, 0,
                                     2 * sizeof(unsigned), b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync(clock)");
-    b->clock_set = true;
+    b->clock_set = runs_now(b);
   }
   int64_t s = 0;
   // The steps before the last: several per launch, as lbm_step takes them

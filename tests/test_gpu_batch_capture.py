@@ -82,3 +82,29 @@ def test_replays_between_calls_of_other_lengths(between):
             assert np.array_equal(x, y)
         got.close()
         want.close()
+
+
+@pytest.mark.parametrize("first", [0, 1])
+def test_lists_of_a_capture_that_never_ran(first):
+    """Work lists that a capture only recorded are uploaded by the next call
+    (the members' block tiles with no call before the capture, their regions
+    with none of three steps or more), and a replay after it finds them too."""
+    import torch
+    from paper_1912_09327_gb300 import binding as b
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        got, doms = make(b, s, "f32", "stochastic")
+        want, other = make(b, s, "f32", "stochastic")
+        if first:
+            got.step(2)
+            want.step(2)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+            got.step(8)
+        got.step(8)
+        want.step(8)
+        for x, y in zip(states(doms), states(other)):
+            assert np.array_equal(x, y)
+        got.close()
+        want.close()

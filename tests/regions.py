@@ -2,7 +2,10 @@
 its C++ names, for tests that say which tiling they cover."""
 import ctypes
 
-from paper_1912_09327_gb300 import binding
+import __graft_entry__
+
+__graft_entry__.build()
+from paper_1912_09327_gb300 import binding  # noqa: E402  (loads the library)
 
 
 class Shape(ctypes.Structure):

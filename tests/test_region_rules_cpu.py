@@ -1,8 +1,6 @@
 """Which domains the region launches serve: the rule alone, without a GPU."""
 import pytest
 
-from . import regions
-
 WIDEST = 1 << 23  # elements per row; the pitch is a caller's (a multiple of 32)
 
 
@@ -11,6 +9,8 @@ WIDEST = 1 << 23  # elements per row; the pitch is a caller's (a multiple of 32)
 def test_pitch_fits_32_bit_offsets(rows, warps):
     """A region's offsets are 32-bit products of a row count and the pitch, so
     a wide pitch leaves the domain to the single-step kernel."""
+    from . import regions
+
     def t(pitch):
         return regions.tiles(regions.shape(100, 90, pitch=pitch), rows, warps, 1)
 
